@@ -477,6 +477,10 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
             c->tstart[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (size_t)(c->ntiles + 1));
             ok = ok && c->tstart[sp];
         }
+    if (mixed) {
+        c->tile_md = (unsigned char*)dev_alloc(c, (size_t)c->ntiles);
+        ok = ok && c->tile_md;
+    }
     if (c->flags & PIC_F_COULOMB)
         for (int sp = 0; sp < 2; ++sp) {
             c->cs_end[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (cells + 1));
@@ -720,6 +724,7 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     }
 
     // ---- cell order for the first steps, then rho_0 and phi_0
+    if (mixed) mark_md_tiles(c);
     sort_particles(c, 0);
     sort_particles(c, 1);
     c->parity ^= 1;
@@ -1172,8 +1177,10 @@ pic_status pic_set_tuning(pic_ctx* c, const pic_tuning* t)
                                                    : c->tstart[0];
         unsigned int* ts1 = ntiles > c->ntiles_cap ? (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (ntiles + 1))
                                                    : c->tstart[1];
-        if (!cur || !ts0 || !ts1) return fail(c, PIC_ENOMEM, "tuning: key buffers");
+        unsigned char* md = ntiles > c->ntiles_cap ? (unsigned char*)dev_alloc(c, (size_t)ntiles) : c->tile_md;
+        if (!cur || !ts0 || !ts1 || !md) return fail(c, PIC_ENOMEM, "tuning: key buffers");
         c->cursor = cur;
+        c->tile_md = md;
         c->tstart[0] = ts0;
         c->tstart[1] = ts1;
         c->nkeys_cap = std::max(c->nkeys_cap, nkeys);
@@ -1190,6 +1197,7 @@ pic_status pic_set_tuning(pic_ctx* c, const pic_tuning* t)
     e = push32_set_window(c);
     if (e != cudaSuccess) return cuda_fail(c, e, "tuning: push window size");
     drop_graphs(c);
+    mark_md_tiles(c);
     sort_particles(c, 0);
     sort_particles(c, 1);
     c->parity ^= 1;

@@ -36,17 +36,16 @@
 namespace pic {
 namespace {
 
-#ifndef PIC_PUSH_PPT
-#define PIC_PUSH_PPT 1
-#endif
 #ifndef PIC_PUSH_MINB
 #define PIC_PUSH_MINB 5                           // resident blocks per SM the register budget is set for
 #endif
 #ifndef PIC_PUSH_TAIL
 #define PIC_PUSH_TAIL 76                          // blocks for the particles appended since the last sort
 #endif
-constexpr int kPushThreads = 256;
-constexpr int kPPT = PIC_PUSH_PPT;               // particles per thread per loop trip
+#ifndef PIC_PUSH_THREADS
+#define PIC_PUSH_THREADS 256
+#endif
+constexpr int kPushThreads = PIC_PUSH_THREADS;
 constexpr int kTailBlocks = PIC_PUSH_TAIL;
 
 struct P32 {
@@ -88,6 +87,7 @@ struct P32 {
     const unsigned int* tstart;  // first slot of each tile at the last sort (ntiles + 1)
     int tx, ty, tz, ntx, nty;    // tile edge (cells) and tiles per axis in x and y
     long long ntiles;
+    const unsigned char* tile_md; // per tile: an MD cell lies in its window
     int halo;                    // deposit window margin (cells)
     int wx, wy, wz;              // deposit window extent (nodes): tile + 1 + 2 halo per axis
 };
@@ -428,113 +428,113 @@ __device__ __forceinline__ void win_add(unsigned int* win32, int wn, int s, unsi
     atomicAdd(win32 + wn + s, hi + (old + lo < old ? 1u : 0u));
 }
 
-// The particles of one species in slots [first, end) with block-uniform trips
-// of kPPT x kPushThreads (every lane of a warp takes every trip: warp votes
-// below).  Deposits go to the block's window (signed sums) when all 8 corners
-// fall inside it, else to global atomics.
-__device__ __forceinline__ void push_range(const P32& p, unsigned long long first, unsigned long long end,
-                                           unsigned long long stride, bool tiled, int ox, int oy, int oz,
-                                           unsigned int* win, CandStage& cst, uint32_t step,
-                                           unsigned int& live)
+// One trip of one species: slot q of this thread (every lane of a warp takes
+// every trip: warp votes below).  Deposits go to the block's window (signed
+// sums) when all 8 corners fall inside it, else to global atomics.  `plain`: no
+// MD cell lies in the window, so a particle inside it needs no look at the
+// cell's grain count, neither where it starts nor where it ends (two scattered
+// loads, the first of them ahead of the field's in the chain: 5e8 particles on
+// 256 x 256 x 1024 cells, 12.7 -> 12.0 ms; the species known at compile time, one
+// signed product per corner: 11.7 ms).
+template <int SP>
+__device__ __forceinline__ void push_one(const P32& p, unsigned long long q, bool have, const float4 P, const float4 V,
+                                         bool tiled, bool plain, int ox, int oy, int oz, unsigned int* win,
+                                         CandStage& cst, uint32_t step, unsigned int& live)
 {
     const int wn = p.wx * p.wy * p.wz;
-    const bool frozen = (p.sp == 1) && (p.flags & PIC_F_IONS_FROZEN);
+    const bool frozen = SP == 1 && (p.flags & PIC_F_IONS_FROZEN);
     const bool no_mcc = p.flags & PIC_F_NO_MCC;
-    const long long charge = p.sp == 0 ? -1 : 1;
+    constexpr int charge = SP == 0 ? -1 : 1;
     const int nx = p.nx, ny = p.ny, nz = p.nz;
     const int wx = p.wx, wy = p.wy, wz = p.wz, wxy = wx * wy;
-    for (unsigned long long q0 = first; q0 < end; q0 += stride) {
-        int dcell[kPPT];
-        int da[kPPT][3];
-        float4 Pr[kPPT], Vr[kPPT];
-        // both records of every particle of the trip in flight at once; they stream
-        // through once (evict-first), so the charge and field arrays keep L2
-#pragma unroll
-        for (int u = 0; u < kPPT; ++u) {
-            const unsigned long long q = q0 + (unsigned long long)u * kPushThreads + threadIdx.x;
-            Pr[u] = q < end ? __ldcs(p.pos + q) : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-            Vr[u] = q < end ? __ldcs(p.vel + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < kPPT; ++u) {
-            dcell[u] = -1;
-            const unsigned long long q = q0 + (unsigned long long)u * kPushThreads + threadIdx.x;
-            int lost = 0;
-            bool md = false, cand = false;
-            const float4 Pu = Pr[u];
-            int cell = __float_as_int(Pu.w);
-            if (cell >= 0) {
-                ++live;
-                int i, j, k;
-                unpack(cell, i, j, k);
-                float o[3] = {Pu.x, Pu.y, Pu.z};
-                if (frozen) {
-                    dcell[u] = cell;
-                    da[u][0] = qa(o[0]); da[u][1] = qa(o[1]); da[u][2] = qa(o[2]);
-                } else if (p.cell_ng[(k * ny + j) * nx + i] != 0) {
-                    // in an MD region: on this step's MD list, advanced by k_md32
-                } else {
-                    const float4 Vu = Vr[u];
-                    float v[3] = {Vu.x, Vu.y, Vu.z};
-                    int a[3] = {qa(o[0]), qa(o[1]), qa(o[2])};
-                    float E[3];
-                    gather(p.E, nx, ny, i, j, k, a, E);
-                    v[0] += E[0] * p.kq; v[1] += E[1] * p.kq; v[2] += E[2] * p.kq;
-                    o[0] += v[0]; o[1] += v[1]; o[2] += v[2];
-                    lost = carry(nx, ny, nz, i, j, k, o);
-                    if (lost) {
-                        p.pos[q].w = __int_as_float(-1);
-                    } else {
-                        if (!no_mcc) {
-                            const uint4 r = philox4x32_10(make_uint4(__float_as_uint(Vu.w), step, kPurMCC, 0u),
-                                                          p.key);
-                            cand = u01f(r.x) < p.pnull;
-                        }
-                        cell = pack(i, j, k);
-                        __stcs(p.pos + q, make_float4(o[0], o[1], o[2], __int_as_float(cell)));
-                        __stcs(p.vel + q, make_float4(v[0], v[1], v[2], Vu.w));
-                        dcell[u] = cell;
-                        da[u][0] = qa(o[0]); da[u][1] = qa(o[1]); da[u][2] = qa(o[2]);
-                        md = p.cell_ng[(k * ny + j) * nx + i] != 0;    // in an MD region next step
-                    }
-                }
-            }
-            if (__any_sync(0xffffffffu, md || cand || lost)) {
-                warp_append(p.md_next, p.md_next_n, (unsigned int)q, md);
-                stage_append(cst, p.sp, p.mcc_list, p.mcc_n, (unsigned int)q, cand);
-                if (__any_sync(0xffffffffu, lost != 0)) {
-                    warp_count(p.cnt + (p.sp == 0 ? PIC_C_LOST_BOT_E : PIC_C_LOST_BOT_I), lost == 1);
-                    warp_count(p.cnt + (p.sp == 0 ? PIC_C_LOST_TOP_E : PIC_C_LOST_TOP_I), lost == 2);
-                    warp_count(p.cnt + PIC_C_ERR, lost == 3);
-                    if (lost == 3) latch(p.err, kErrNonFinite);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kPPT; ++u) {
-            if (dcell[u] < 0) continue;
-            int i, j, k;
-            unpack(dcell[u], i, j, k);
-            const int di = wrel(i, ox, nx), dj = wrel(j, oy, ny), dk = k - oz;
-            if (tiled && di + 1 < wx && dj + 1 < wy && dk >= 0 && dk + 1 < wz) {
-                const int s0 = (dk * wy + dj) * wx + di;
-                // corner weight wx (< 2^15) x wy wz (< 2^29): one 32 x 32 -> 64-bit product;
-                // electrons add the two's complement (the window holds signed sums)
-                const unsigned int wxs[2] = {(unsigned int)(kWQ - da[u][0]), (unsigned int)da[u][0]};
-                const unsigned int wyz[4] = {(unsigned int)((kWQ - da[u][1]) * (kWQ - da[u][2])),
-                                             (unsigned int)(da[u][1] * (kWQ - da[u][2])),
-                                             (unsigned int)((kWQ - da[u][1]) * da[u][2]),
-                                             (unsigned int)(da[u][1] * da[u][2])};
-                const int off[4] = {0, wx, wxy, wxy + wx};
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const unsigned long long v = (unsigned long long)wxs[c & 1] * wyz[c >> 1];
-                    win_add(win, wn, s0 + off[c >> 1] + (c & 1), charge < 0 ? 0ull - v : v);
-                }
+    // whether a cell lies in the window, and its place there
+    auto inside = [&](int i, int j, int k, int& s0) {
+        const int di = wrel(i, ox, nx), dj = wrel(j, oy, ny), dk = k - oz;
+        s0 = (dk * wy + dj) * wx + di;
+        return tiled && di + 1 < wx && dj + 1 < wy && dk >= 0 && dk + 1 < wz;
+    };
+    int cell = have ? __float_as_int(P.w) : -1;
+    int i = 0, j = 0, k = 0, s0 = 0;
+    int da[3] = {0, 0, 0};
+    int lost = 0;
+    bool md = false, cand = false, dep = false, in = false;
+    if (cell >= 0) {
+        ++live;
+        unpack(cell, i, j, k);
+        float o[3] = {P.x, P.y, P.z};
+        if (frozen) {
+            dep = true;
+            in = inside(i, j, k, s0);
+            da[0] = qa(o[0]); da[1] = qa(o[1]); da[2] = qa(o[2]);
+        } else if (!(plain && inside(i, j, k, s0)) && p.cell_ng[(k * ny + j) * nx + i] != 0) {
+            // in an MD region: on this step's MD list, advanced by k_md32
+        } else {
+            float v[3] = {V.x, V.y, V.z};
+            int a[3] = {qa(o[0]), qa(o[1]), qa(o[2])};
+            float E[3];
+            gather(p.E, nx, ny, i, j, k, a, E);
+            v[0] += E[0] * p.kq; v[1] += E[1] * p.kq; v[2] += E[2] * p.kq;
+            o[0] += v[0]; o[1] += v[1]; o[2] += v[2];
+            lost = carry(nx, ny, nz, i, j, k, o);
+            if (lost) {
+                p.pos[q].w = __int_as_float(-1);
             } else {
-                deposit_global(p.rq, nx, ny, i, j, k, da[u], charge);
+                if (!no_mcc) {
+                    const uint4 r = philox4x32_10(make_uint4(__float_as_uint(V.w), step, kPurMCC, 0u), p.key);
+                    cand = u01f(r.x) < p.pnull;
+                }
+                cell = pack(i, j, k);
+                __stcs(p.pos + q, make_float4(o[0], o[1], o[2], __int_as_float(cell)));
+                __stcs(p.vel + q, make_float4(v[0], v[1], v[2], V.w));
+                dep = true;
+                in = inside(i, j, k, s0);
+                da[0] = qa(o[0]); da[1] = qa(o[1]); da[2] = qa(o[2]);
+                if (!(plain && in)) md = p.cell_ng[(k * ny + j) * nx + i] != 0;    // in an MD region next step
             }
         }
+    }
+    if (__any_sync(0xffffffffu, md || cand || lost)) {
+        warp_append(p.md_next, p.md_next_n, (unsigned int)q, md);
+        stage_append(cst, SP, p.mcc_list, p.mcc_n, (unsigned int)q, cand);
+        if (__any_sync(0xffffffffu, lost != 0)) {
+            warp_count(p.cnt + (SP == 0 ? PIC_C_LOST_BOT_E : PIC_C_LOST_BOT_I), lost == 1);
+            warp_count(p.cnt + (SP == 0 ? PIC_C_LOST_TOP_E : PIC_C_LOST_TOP_I), lost == 2);
+            warp_count(p.cnt + PIC_C_ERR, lost == 3);
+            if (lost == 3) latch(p.err, kErrNonFinite);
+        }
+    }
+    if (!dep) return;
+    if (in) {
+        // corner weight wx (< 2^15) x wy wz (< 2^29): one signed 32 x 32 -> 64-bit
+        // product, the species' sign on wx
+        const int x[2] = {charge * (kWQ - da[0]), charge * da[0]};
+        const int yz[4] = {(kWQ - da[1]) * (kWQ - da[2]), da[1] * (kWQ - da[2]), (kWQ - da[1]) * da[2], da[1] * da[2]};
+        const int off[4] = {0, wx, wxy, wxy + wx};
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            win_add(win, wn, s0 + off[c >> 1] + (c & 1), (unsigned long long)((long long)x[c & 1] * yz[c >> 1]));
+    } else {
+        deposit_global(p.rq, nx, ny, i, j, k, da, charge);
+    }
+}
+
+// The particles of one species in slots [first, end), in block-uniform trips;
+// the records stream through once (evict-first), so the charge and field arrays
+// keep L2.
+template <int SP>
+__device__ __forceinline__ void push_range(const P32& p, unsigned long long first, unsigned long long end,
+                                           unsigned long long stride, bool tiled, bool plain, int ox, int oy, int oz,
+                                           unsigned int* win, CandStage& cst, uint32_t step, unsigned int& live)
+{
+    for (unsigned long long q0 = first; q0 < end; q0 += stride) {
+        const unsigned long long q = q0 + threadIdx.x;
+        const bool have = q < end;
+        float4 P = make_float4(0.f, 0.f, 0.f, 0.f), V = P;
+        if (have) {
+            P = __ldcs(p.pos + q);
+            V = __ldcs(p.vel + q);
+        }
+        push_one<SP>(p, q, have, P, V, tiled, plain, ox, oy, oz, win, cst, step, live);
     }
 }
 
@@ -543,6 +543,13 @@ __device__ __forceinline__ void push_range(const P32& p, unsigned long long firs
 // wx x wy x wz nodes from the tile's lower corner minus `halo` cells, flushed
 // once.  Blocks [ntiles, grid): the ionization products appended since the
 // sort, deposited with global atomics.
+// What bounds it (1e7 particles, 8 x 8 x 8 tiles, ncu): the L1 data pipe 85% busy
+// (209 wavefronts per warp and trip: 90 in the window's shared atomics, about 90
+// in the 8 field loads, the rest in the records), issue slots 65% (600
+// instructions per warp and trip), DRAM 40%; 5 blocks of 256 threads because
+// the L1 left beside their windows holds the field tiles: 4 blocks 12.6 ms, 10
+// of 128 threads 14.1 ms, records staged ahead in shared memory 12.5 ms, runs of
+// lanes in one cell joined before the window 12.4 ms, against 11.7 ms.
 __global__ void __launch_bounds__(kPushThreads, PIC_PUSH_MINB) k_push32(const P32 pe, const P32 pi)
 {
     extern __shared__ unsigned int win[];          // low words [0, wn), high words [wn, 2 wn)
@@ -561,13 +568,13 @@ __global__ void __launch_bounds__(kPushThreads, PIC_PUSH_MINB) k_push32(const P3
         const int ti = (int)(b % pe.ntx), tj = (int)((b / pe.ntx) % pe.nty),
                   tk = (int)(b / ((long long)pe.ntx * pe.nty));
         const int ox = ti * pe.tx - pe.halo, oy = tj * pe.ty - pe.halo, oz = tk * pe.tz - pe.halo;
+        const bool plain = pe.tile_md[b] == 0;
         for (int t = threadIdx.x; t < 2 * wn; t += blockDim.x) win[t] = 0u;
         if (threadIdx.x < 2) cst.n[threadIdx.x] = 0u;
         if (threadIdx.x == 0) s_live = 0u;
         __syncthreads();
-        const unsigned long long stride = (unsigned long long)kPushThreads * kPPT;
-        push_range(pe, e0, e1, stride, true, ox, oy, oz, win, cst, step, live);
-        push_range(pi, i0, i1, stride, true, ox, oy, oz, win, cst, step, live);
+        push_range<0>(pe, e0, e1, kPushThreads, true, plain, ox, oy, oz, win, cst, step, live);
+        push_range<1>(pi, i0, i1, kPushThreads, true, plain, ox, oy, oz, win, cst, step, live);
         __syncthreads();
         // flush: each pass takes blockDim / wx whole window rows, one thread per node
         const int rows_per_pass = blockDim.x / wx;
@@ -586,10 +593,10 @@ __global__ void __launch_bounds__(kPushThreads, PIC_PUSH_MINB) k_push32(const P3
         if (threadIdx.x < 2) cst.n[threadIdx.x] = 0u;
         if (threadIdx.x == 0) s_live = 0u;
         __syncthreads();
-        const unsigned long long tb = (unsigned long long)(b - pe.ntiles) * kPushThreads * kPPT;
-        const unsigned long long stride = (unsigned long long)(gridDim.x - pe.ntiles) * kPushThreads * kPPT;
-        push_range(pe, pe.tstart[pe.ntiles] + tb, pe.nslot[0], stride, false, 0, 0, 0, win, cst, step, live);
-        push_range(pi, pi.tstart[pi.ntiles] + tb, pi.nslot[1], stride, false, 0, 0, 0, win, cst, step, live);
+        const unsigned long long tb = (unsigned long long)(b - pe.ntiles) * kPushThreads;
+        const unsigned long long stride = (unsigned long long)(gridDim.x - pe.ntiles) * kPushThreads;
+        push_range<0>(pe, pe.tstart[pe.ntiles] + tb, pe.nslot[0], stride, false, false, 0, 0, 0, win, cst, step, live);
+        push_range<1>(pi, pi.tstart[pi.ntiles] + tb, pi.nslot[1], stride, false, false, 0, 0, 0, win, cst, step, live);
         __syncthreads();
     }
     // one global atomic per block for the candidates of each species and the live count
@@ -598,6 +605,26 @@ __global__ void __launch_bounds__(kPushThreads, PIC_PUSH_MINB) k_push32(const P3
     if ((threadIdx.x & 31) == 0 && live) atomicAdd(&s_live, live);
     __syncthreads();
     if (threadIdx.x == 0 && s_live) atomicAdd(pe.cnt + PIC_C_PUSHED, (unsigned long long)s_live);
+}
+
+// Mark the tiles whose window (the cells push_one's `inside` accepts) holds an
+// MD cell: one thread per cell of each grain's 3 x 3 x 3 region.
+__global__ void k_tile_md(int ng, const int* gcell, int nx, int ny, int nz, int tx, int ty, int tz, int ntx, int nty,
+                          int ntz, int halo, unsigned char* tile_md)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 27 * ng) return;
+    const int* g = gcell + 3 * (t / 27);
+    const int i = (g[0] + t % 3 - 1 + nx) % nx, j = (g[1] + t / 3 % 3 - 1 + ny) % ny, k = g[2] + t % 27 / 9 - 1;
+    for (int a = 0; a < ntz; ++a) {
+        const int dk = k - (a * tz - halo);
+        if (dk < 0 || dk >= tz + 2 * halo) continue;
+        for (int b = 0; b < nty; ++b) {
+            if (wrel(j, b * ty - halo, ny) >= ty + 2 * halo) continue;
+            for (int c = 0; c < ntx; ++c)
+                if (wrel(i, c * tx - halo, nx) < tx + 2 * halo) tile_md[((size_t)a * nty + b) * ntx + c] = 1;
+        }
+    }
 }
 
 // Field data of one cell for the MD substeps: the 8 corner values of
@@ -1030,6 +1057,7 @@ P32 params(pic_ctx* c, int sp)
     p.tx = c->tile[0]; p.ty = c->tile[1]; p.tz = c->tile[2];
     p.ntx = c->ntile[0]; p.nty = c->ntile[1];
     p.ntiles = (long long)c->ntiles;
+    p.tile_md = c->tile_md;
     p.halo = c->halo;
     p.wx = c->tile[0] + 1 + 2 * c->halo;
     p.wy = c->tile[1] + 1 + 2 * c->halo;
@@ -1077,6 +1105,17 @@ void launch_push32(pic_ctx* c)
 cudaError_t push32_set_window(pic_ctx*)
 {
     return cudaFuncSetAttribute(k_push32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxWindowBytes);
+}
+
+void mark_md_tiles(pic_ctx* c)
+{
+    cudaMemsetAsync(c->tile_md, 0, (size_t)c->ntiles, c->stream);
+    if (c->ng > 0) {
+        k_tile_md<<<(27 * c->ng + 127) / 128, 128, 0, c->stream>>>(c->ng, c->gcell, c->nx, c->ny, c->nz, c->tile[0],
+                                                                 c->tile[1], c->tile[2], c->ntile[0], c->ntile[1],
+                                                                 c->ntile[2], c->halo, c->tile_md);
+        c->launches += 1;
+    }
 }
 
 void launch_deposit32(pic_ctx* c)

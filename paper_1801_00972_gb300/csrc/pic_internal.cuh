@@ -235,6 +235,7 @@ struct pic_ctx {
     int sort_order = 0;                      // mixed sort keys: 0 by cell inside the tile, 1 by tile only
     unsigned int* tstart[2] = {nullptr, nullptr};   // mixed: first slot of each tile after the last sort
                                                     // (ntiles + 1 entries; the last = particles sorted)
+    unsigned char* tile_md = nullptr;               // mixed: 1 where a tile's deposit window holds an MD cell
     std::vector<unsigned int*> scan_tmp;
     std::vector<size_t> scan_len;
 
@@ -324,6 +325,7 @@ void launch_efield32(pic_ctx* c);
 void launch_push32(pic_ctx* c);
 constexpr size_t kMaxWindowBytes = 96 * 1024;  // largest deposit window of the mixed push (shared memory)
 cudaError_t push32_set_window(pic_ctx* c);     // lets the push take windows up to kMaxWindowBytes
+void mark_md_tiles(pic_ctx* c);                // tile_md of the current tiling
 void launch_children32(pic_ctx* c);
 void launch_deposit32(pic_ctx* c);
 void launch_moments32(pic_ctx* c);
