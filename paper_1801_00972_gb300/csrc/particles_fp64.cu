@@ -7,18 +7,32 @@
 // This translation unit is compiled with --fmad=false: every product and sum
 // rounds on its own, in the order written, so an FP64 step on the GPU is
 // bit-identical to a plain FP64 CPU evaluation of the same formulas.
+#include <algorithm>
+#include <cmath>
+
 #include "pic_internal.cuh"
 
 namespace pic {
 namespace {
 
-struct P64 {
+struct Geo {
     int nx, ny, nz;
     double dx, Lx, Ly, Lz;
+    double rdx;                  // 1 / dx rounded to nearest, or 0: divide
+    unsigned long long fix_c;    // 1 / dx = fix_c 2^(-63 - fix_e), fix_c rounded down (0: not used, see fix_cell)
+    int fix_e;
+};
+
+struct P64 {
+    Geo g;
+    double Lx, Ly;
     double dt, dtm;
     int M;
     int sp;
-    double qmdt, qmdtm, hm, pnull, nu_max, de;
+    double qmdt, qmdtm, hm, nu_max, de;
+    unsigned long long null_below;   // a particle collides if its 32-bit draw is below this
+    unsigned int* mcc_list;      // slots of this step's collision candidates
+    unsigned int* mcc_n;
     double n_gas, sig_n, eps_exc, eps_ion, mr2, kc;
     int n_xs;
     const double* xs;
@@ -48,18 +62,27 @@ struct P64 {
     unsigned long long* nch;
 };
 
-struct Geo {
-    int nx, ny, nz;
-    double dx, Lx, Ly, Lz;
-};
+// x / dx, correctly rounded, from the rounded reciprocal: two residual
+// corrections by fused multiply-adds (Markstein, IBM J. Res. Dev. 34, 1990: with
+// y = RN(1 / b) and q within an ulp of a / b, RN(q + y RN(a - b q)) is the
+// correctly rounded quotient; the first correction brings q there).  5 FP64
+// instructions, where the pipe issues one every 16 cycles per warp and a
+// particle divides six times.
+__device__ __forceinline__ double over_dx(const Geo& g, double x)
+{
+    if (g.rdx == 0.0) return x / g.dx;
+    double q = x * g.rdx;
+    q = fma(fma(-q, g.dx, x), g.rdx, q);
+    return fma(fma(-q, g.dx, x), g.rdx, q);
+}
 
 __device__ __forceinline__ void locate(const Geo& g, const double x[3], int c[3], double f[3])
 {
     const int nn[3] = {g.nx, g.ny, g.nz};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const double q = x[a] / g.dx;
-        int i = (int)floor(q);
+        const double q = over_dx(g, x[a]);
+        int i = __double2int_rd(q);
         if (i > nn[a] - 1) i = nn[a] - 1;
         if (i < 0) i = 0;
         c[a] = i;
@@ -67,57 +90,162 @@ __device__ __forceinline__ void locate(const Geo& g, const double x[3], int c[3]
     }
 }
 
-__device__ __forceinline__ void qweights(const double f[3], long long w[3][2])
-{
+// Fixed-point CIC weights: per axis a = round_half_even(f 2^14) in [0, 2^14] as an
+// integer (deposit) and the pair (1 - a 2^-14, a 2^-14) in FP64 (gather; the
+// products of three are exact).  The rounding is the sum with 1.5 2^52, whose
+// last place is 1 and whose low word then holds the integer: no conversion.
+struct Cic {
+    int a[3];
+    double w[3][2];
+    __device__ __forceinline__ explicit Cic(const double f[3])
+    {
+        const double big = 6755399441055744.0;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        long long q = (long long)rint(f[a] * (double)kWQ);
-        if (q < 0) q = 0;
-        if (q > kWQ) q = kWQ;
-        w[a][0] = kWQ - q;
-        w[a][1] = q;
+        for (int d = 0; d < 3; ++d) {
+            const double t = f[d] * (double)kWQ + big;
+            int q = __double2loint(t);
+            double u = t - big;
+            if (!(u >= 0.0)) { q = 0; u = 0.0; }
+            if (u > (double)kWQ) { q = kWQ; u = (double)kWQ; }
+            a[d] = q;
+            w[d][1] = u * (1.0 / (double)kWQ);
+            w[d][0] = 1.0 - w[d][1];
+        }
     }
+};
+
+// Cell i and weight a of one coordinate in integer arithmetic: the FP64 pipe
+// issues a warp instruction every 16 cycles and SM, the integer pipes two a
+// cycle, so 30 integer instructions are cheaper than the 14 FP64 ones of
+// locate and Cic.  With q = RN(x / dx), i = floor(q) and
+// a = round_half_even((q - i) 2^14) (q - i is exact).  Here Y = x / dx 2^46 as an
+// integer, off by at most 3 (the reciprocal and the product are each cut once),
+// and q 2^46 itself is within 2^-53 x / dx 2^46 <= 2^9 of the exact quotient for
+// x / dx < 2^16: unless Y lies within 2^12 of a cell boundary or of a tie, both
+// results are those of any number within that distance, q among them.  Returns
+// false there (one coordinate in 5e5, and coordinates on nodes), at x = 0, and
+// for x / dx >= 2^16.
+__device__ __forceinline__ bool fix_cell(const Geo& g, double x, int& i, int& a)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int E = (int)(b >> 52);                                // x >= 0: the biased exponent
+    const unsigned long long m = ((b << 11) | (1ull << 63));     // significand, leading one made explicit
+    const int sh = 1039 + g.fix_e - E;
+    if (sh < 1 || sh > 63) return false;
+    const unsigned long long Y = __umul64hi(m, g.fix_c) >> sh;
+    const unsigned int hi = (unsigned int)(Y >> 32), lo = (unsigned int)Y;
+    const unsigned long long t = Y + 4096ull;
+    if (lo - 0x80000000u + 4096u < 8192u || ((((unsigned int)(t >> 32)) & 0x3fffu) == 0u && (unsigned int)t < 8192u))
+        return false;
+    i = (int)(hi >> 14);
+    a = (int)((hi + (lo >> 31)) - ((unsigned int)i << 14));
+    return true;
 }
 
-__device__ __forceinline__ size_t node_at(const Geo& g, int i, int j, int k)
+__device__ __noinline__ void exact_cell(const Geo& g, const double x[3], int c[3], int a[3])
 {
-    i %= g.nx;
-    j %= g.ny;
-    return ((size_t)k * g.ny + j) * g.nx + i;
+    double f[3];
+    locate(g, x, c, f);
+    const Cic w(f);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) a[d] = w.a[d];
+}
+
+// cell and integer weights of a position
+__device__ __forceinline__ void cell_weights(const Geo& g, const double x[3], int c[3], int a[3])
+{
+    bool ok = g.fix_c != 0ull;
+    if (ok)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) ok = fix_cell(g, x[d], c[d], a[d]) && ok;
+    if (!ok) exact_cell(g, x, c, a);
+}
+
+// n as a double, 0 <= n < 2^53, by integer instructions
+__device__ __forceinline__ double exact_double(unsigned long long n)
+{
+    const int e = 63 - __clzll((long long)n);
+    return n ? __longlong_as_double((long long)(((unsigned long long)(1022 + e) << 52) + (n << (52 - e)))) : 0.0;
+}
+__device__ __forceinline__ double exact_double32(unsigned int n)   // n < 2^20: the high word alone
+{
+    const int e = 31 - __clz((int)n);
+    return n ? __hiloint2double((int)(((unsigned int)(1022 + e) << 20) + (n << (20 - e))), 0) : 0.0;
+}
+// a whole number 0 <= v < 2^32
+__device__ __forceinline__ unsigned int exact_uint(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) - 1023;
+    return e < 0 ? 0u : (unsigned int)(((b & ((1ull << 52) - 1ull)) | (1ull << 52)) >> (52 - e));
+}
+
+// node index of the cell's corner (di, dy, dz), periodic in x and y
+__device__ __forceinline__ unsigned int corner(const Geo& g, const int c[3], int di, int dy, int dz)
+{
+    const int i = c[0] + di == g.nx ? 0 : c[0] + di, j = c[1] + dy == g.ny ? 0 : c[1] + dy;
+    return ((unsigned int)(c[2] + dz) * g.ny + j) * g.nx + i;
 }
 
 __device__ __forceinline__ int cell_of(const Geo& g, const int c[3]) { return (c[2] * g.ny + c[1]) * g.nx + c[0]; }
 
-__device__ __forceinline__ void deposit(const Geo& g, unsigned long long* rq, const int c[3], const long long w[3][2],
-                                        long long charge)
+__device__ __forceinline__ void deposit(const Geo& g, unsigned long long* rq, const int c[3], const int a[3], int charge)
 {
+    const int x[2] = {charge * (kWQ - a[0]), charge * a[0]};
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
+        for (int dy = 0; dy < 2; ++dy) {
+            const int yz = (dy ? a[1] : kWQ - a[1]) * (dz ? a[2] : kWQ - a[2]);
 #pragma unroll
             for (int di = 0; di < 2; ++di) {
-                const long long v = charge * (w[0][di] * w[1][dy] * w[2][dz]);
-                if (v != 0) atomicAdd(rq + node_at(g, c[0] + di, c[1] + dy, c[2] + dz), (unsigned long long)v);
+                const long long v = (long long)x[di] * yz;
+                if (v != 0) atomicAdd(rq + corner(g, c, di, dy, dz), (unsigned long long)v);
             }
+        }
 }
 
 __device__ __forceinline__ void gather(const Geo& g, const double* fx, const double* fy, const double* fz,
-                                       const int c[3], const long long w[3][2], double E[3])
+                                       const int c[3], const Cic& w, double E[3])
 {
     E[0] = 0.0; E[1] = 0.0; E[2] = 0.0;
 #pragma unroll
     for (int dz = 0; dz < 2; ++dz)
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
+        for (int dy = 0; dy < 2; ++dy) {
+            const double yz = w.w[1][dy] * w.w[2][dz];
 #pragma unroll
             for (int di = 0; di < 2; ++di) {
-                const double wt = (double)(w[0][di] * w[1][dy] * w[2][dz]) * 0x1p-42;
-                const size_t n = node_at(g, c[0] + di, c[1] + dy, c[2] + dz);
+                const double wt = w.w[0][di] * yz;
+                const unsigned int n = corner(g, c, di, dy, dz);
                 E[0] = E[0] + wt * fx[n];
                 E[1] = E[1] + wt * fy[n];
                 E[2] = E[2] + wt * fz[n];
             }
+        }
+}
+
+// The same gather times 2^42, from the integer weights: the products of three are
+// whole numbers, exact in FP64, and the scale is a power of two, so every sum
+// rounds as in `gather`.
+__device__ __forceinline__ void gather_scaled(const Geo& g, const double* fx, const double* fy, const double* fz,
+                                              const int c[3], const int a[3], double E[3])
+{
+    E[0] = 0.0; E[1] = 0.0; E[2] = 0.0;
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 2; ++dy) {
+            const unsigned int yz = (unsigned int)((dy ? a[1] : kWQ - a[1]) * (dz ? a[2] : kWQ - a[2]));
+#pragma unroll
+            for (int di = 0; di < 2; ++di) {
+                const double wt = exact_double((unsigned long long)(unsigned int)(di ? a[0] : kWQ - a[0]) * yz);
+                const unsigned int n = corner(g, c, di, dy, dz);
+                E[0] = E[0] + wt * fx[n];
+                E[1] = E[1] + wt * fy[n];
+                E[2] = E[2] + wt * fz[n];
+            }
+        }
 }
 
 __device__ __forceinline__ void grain_sep(const P64& p, int gi, const double x[3], double d[3])
@@ -135,8 +263,7 @@ __device__ __forceinline__ void grain_sep(const P64& p, int gi, const double x[3
 
 // E = E_PIC - Q g(x) + Q (x - x_g) / (4 pi eps0 |x - x_g|^3) for the grains whose
 // MD region holds the particle's cell (Eqs. 5-6)
-__device__ void md_correct(const P64& p, const Geo& g, const double x[3], const int c[3], const long long w[3][2],
-                           double E[3])
+__device__ void md_correct(const P64& p, const Geo& g, const double x[3], const int c[3], const Cic& w, double E[3])
 {
     const int cell = cell_of(g, c);
     const int n = p.cell_ng[cell];
@@ -147,7 +274,7 @@ __device__ void md_correct(const P64& p, const Geo& g, const double x[3], const 
         for (int dz = 0; dz < 2; ++dz)
             for (int dy = 0; dy < 2; ++dy)
                 for (int di = 0; di < 2; ++di) {
-                    const double wt = (double)(w[0][di] * w[1][dy] * w[2][dz]) * 0x1p-42;
+                    const double wt = w.w[0][di] * (w.w[1][dy] * w.w[2][dz]);
                     const int li = ((c[0] + di - gc0 + 1) % g.nx + g.nx) % g.nx;
                     const int lj = ((c[1] + dy - gc1 + 1) % g.ny + g.ny) % g.ny;
                     const int lk = c[2] + dz - gc2 + 1;
@@ -170,16 +297,22 @@ __device__ void md_correct(const P64& p, const Geo& g, const double x[3], const 
     }
 }
 
-// 0 alive, 1 lost at z = 0, 2 lost at z = Lz, 3 invalid
+// 0 alive, 1 lost at z = 0, 2 lost at z = Lz, 3 invalid; the comparisons on the
+// bits (ordered as the values from +0 up)
 __device__ __forceinline__ int boundary(const Geo& g, double x[3])
 {
-    if (!(x[2] >= 0.0)) return (x[2] < 0.0) ? 1 : 3;
-    if (x[2] > g.Lz) return 2;
+    const long long inf = 0x7ff0000000000000ll, minus0 = (long long)0x8000000000000000ull;
+    const long long z = __double_as_longlong(x[2]);
+    if ((z & 0x7fffffffffffffffll) > inf) return 3;
+    if (z < 0 && z != minus0) return 1;
+    if (z > __double_as_longlong(g.Lz)) return 2;
     const double L[2] = {g.Lx, g.Ly};
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        if (x[a] < 0.0) x[a] = x[a] + L[a];
-        else if (x[a] >= L[a]) x[a] = x[a] - L[a];
+        const long long b = __double_as_longlong(x[a]);
+        const bool below = b < 0 && b != minus0;
+        if (!below && b < __double_as_longlong(L[a])) continue;
+        x[a] = below ? x[a] + L[a] : x[a] - L[a];
         if (!(x[a] >= 0.0 && x[a] <= L[a])) return 3;
     }
     return 0;
@@ -259,11 +392,10 @@ __device__ void gauss3(RStream& r, double o[3])
 
 __device__ __forceinline__ void latch(int* err, int code) { atomicCAS(err, 0, code); }
 
-// null-collision MCC after the push (Table I); may record an ionization product
-__device__ void mcc(const P64& p, uint32_t step, const double x[3], double v[3], uint32_t id, int cell)
+// process choice and kinematics of a collision candidate (Table I); u = its
+// Philox draw; may record an ionization product
+__device__ void mcc(const P64& p, uint32_t step, uint4 u, const double x[3], double v[3], uint32_t id, int cell)
 {
-    const uint4 u = philox4x32_10(make_uint4(id, step, kPurMCC, 0u), p.key);
-    if (u01d(u.x) >= p.pnull) return;
     const double ng = p.n_gas;
     const int nx = p.n_xs;
     if (p.sp == 0) {
@@ -352,50 +484,62 @@ __device__ void mcc(const P64& p, uint32_t step, const double x[3], double v[3],
     }
 }
 
-__global__ void k_push64(const P64 p)
+// One step of every particle of both species (blockIdx.y): gather, push (MD
+// particles with their substeps), absorption, the null-collision test and the
+// deposit.  The few per cent that pass the test are listed for k_mcc64: their
+// collision, a long chain of FP64 divisions and roots, would otherwise run in
+// almost every warp with one or two lanes active.
+// FP64 bound: the pipe issues one warp instruction per 16 cycles and SM, so what
+// counts is FP64 instructions per particle: 75, of which the gather's products
+// and sums are 48 (each rounds on its own) and the push 12; cells, weights,
+// comparisons and the null test are integer work (fix_cell, exact_double,
+// boundary).  5e6 particles per species, one launch for both: 2 x 2.42 -> 1.98 ms
+// (with the collisions listed and divisions as products only, 163 FP64
+// instructions, 3.99 ms), the pipe 73% active.  5 blocks per SM: 1.98 ms, 3 (all
+// registers) 2.00, 8 2.06.
+constexpr int kPush64Threads = 128;
+constexpr int kCand64 = 512;   // candidates a block stages before they go to the list one by one
+
+__global__ void __launch_bounds__(kPush64Threads, 5) k_push64(const P64 pe, const P64 pi)
 {
-    const Geo g{p.nx, p.ny, p.nz, p.dx, p.Lx, p.Ly, p.Lz};
+    __shared__ unsigned int s_n, s_base, s_cand[kCand64];
+    const P64& p = blockIdx.y == 0 ? pe : pi;
+    const Geo& g = p.g;
     const unsigned long long n = p.nslot[p.sp];
     const uint32_t step = *p.step;
     const bool frozen = (p.sp == 1) && (p.flags & PIC_F_IONS_FROZEN);
-    const long long charge = p.sp == 0 ? -1 : 1;
+    const int charge = p.sp == 0 ? -1 : 1;
     unsigned int live = 0;
+    if (threadIdx.x == 0) s_n = 0u;
+    __syncthreads();
     for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; q < n;
          q += (unsigned long long)gridDim.x * blockDim.x) {
         double4 P = p.pos[q];
-        if (P.w < 0.0) continue;
+        if (__double2hiint(P.w) < 0) continue;   // dead: -1
         ++live;
         double x[3] = {P.x, P.y, P.z};
-        int c[3];
-        double f[3];
-        long long w[3][2];
+        int c[3], ci[3];
+        cell_weights(g, x, c, ci);
         if (frozen) {
-            locate(g, x, c, f);
-            qweights(f, w);
-            deposit(g, p.rq, c, w, charge);
+            deposit(g, p.rq, c, ci, charge);
             continue;
         }
         const double4 V = p.vel[q];
         double v[3] = {V.x, V.y, V.z};
-        const uint32_t id = (uint32_t)V.w;
-        locate(g, x, c, f);
-        qweights(f, w);
         int fate = 0, grain = -1;
         if (p.cell_ng[cell_of(g, c)] == 0) {
             double E[3];
-            gather(g, p.ex, p.ey, p.ez, c, w, E);
+            gather_scaled(g, p.ex, p.ey, p.ez, c, ci, E);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) v[a] = v[a] + p.qmdt * E[a];
+            for (int a = 0; a < 3; ++a) v[a] = v[a] + p.qmdt * E[a];   // (qmdt carries the 2^-42)
 #pragma unroll
             for (int a = 0; a < 3; ++a) x[a] = x[a] + v[a] * p.dt;
             fate = boundary(g, x);
         } else {
             for (int m = 0; m < p.M; ++m) {
-                double E[3];
-                if (m > 0) {
-                    locate(g, x, c, f);
-                    qweights(f, w);
-                }
+                double E[3], f[3];
+                locate(g, x, c, f);
+                const Cic w(f);
                 gather(g, p.ex, p.ey, p.ez, c, w, E);
                 md_correct(p, g, x, c, w, E);
 #pragma unroll
@@ -421,16 +565,45 @@ __global__ void k_push64(const P64 p)
             }
             continue;
         }
-        locate(g, x, c, f);
-        const int cell = cell_of(g, c);
-        if (!(p.flags & PIC_F_NO_MCC)) mcc(p, step, x, v, id, cell);
-        p.pos[q] = make_double4(x[0], x[1], x[2], (double)cell);
-        p.vel[q] = make_double4(v[0], v[1], v[2], (double)id);
-        qweights(f, w);
-        deposit(g, p.rq, c, w, charge);
+        cell_weights(g, x, c, ci);
+        if (!(p.flags & PIC_F_NO_MCC)) {
+            const uint4 u = philox4x32_10(make_uint4(exact_uint(V.w), step, kPurMCC, 0u), p.key);
+            // (u + 1/2) 2^-32 < pnull, both sides exact
+            if ((unsigned long long)u.x < p.null_below) {
+                const unsigned int at = atomicAdd(&s_n, 1u);
+                if (at < kCand64) s_cand[at] = (unsigned int)q;
+                else p.mcc_list[atomicAdd(p.mcc_n, 1u)] = (unsigned int)q;
+            }
+        }
+        p.pos[q] = make_double4(x[0], x[1], x[2], exact_double((unsigned long long)(unsigned int)cell_of(g, c)));
+        p.vel[q] = make_double4(v[0], v[1], v[2], V.w);
+        deposit(g, p.rq, c, ci, charge);
     }
     live = __reduce_add_sync(0xffffffffu, live);
     if ((threadIdx.x & 31) == 0 && live) atomicAdd(p.cnt + PIC_C_PUSHED, (unsigned long long)live);
+    __syncthreads();
+    const unsigned int k = min(s_n, (unsigned int)kCand64);
+    if (threadIdx.x == 0 && k) s_base = atomicAdd(p.mcc_n, k);
+    __syncthreads();
+    for (unsigned int t = threadIdx.x; t < k; t += blockDim.x) p.mcc_list[s_base + t] = s_cand[t];
+}
+
+// the listed collision candidates of both species (blockIdx.y), after the push
+__global__ void __launch_bounds__(kPush64Threads) k_mcc64(const P64 pe, const P64 pi)
+{
+    const P64& p = blockIdx.y == 0 ? pe : pi;
+    const unsigned int n = *p.mcc_n;
+    const uint32_t step = *p.step;
+    for (unsigned int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+        const unsigned int q = p.mcc_list[t];
+        const double4 P = p.pos[q], V = p.vel[q];
+        const uint32_t id = (uint32_t)V.w;
+        const uint4 u = philox4x32_10(make_uint4(id, step, kPurMCC, 0u), p.key);
+        const double x[3] = {P.x, P.y, P.z};
+        double v[3] = {V.x, V.y, V.z};
+        mcc(p, step, u, x, v, id, (int)P.w);
+        p.vel[q] = make_double4(v[0], v[1], v[2], V.w);
+    }
 }
 
 // deposit every live particle (initial rho and re-deposits)
@@ -438,7 +611,7 @@ __global__ void k_deposit64(Geo g, const double4* pos, const unsigned long long*
                             unsigned long long* rq)
 {
     const unsigned long long n = nslot[sp];
-    const long long charge = sp == 0 ? -1 : 1;
+    const int charge = sp == 0 ? -1 : 1;
     for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; q < n;
          q += (unsigned long long)gridDim.x * blockDim.x) {
         const double4 P = pos[q];
@@ -446,10 +619,8 @@ __global__ void k_deposit64(Geo g, const double4* pos, const unsigned long long*
         const double x[3] = {P.x, P.y, P.z};
         int c[3];
         double f[3];
-        long long w[3][2];
         locate(g, x, c, f);
-        qweights(f, w);
-        deposit(g, rq, c, w, charge);
+        deposit(g, rq, c, Cic(f).a, charge);
     }
 }
 
@@ -512,16 +683,15 @@ __global__ void k_children64(Geo g, ChildRec* rec, const unsigned long long* nch
         const double x[3] = {cr.x[0], cr.x[1], cr.x[2]};
         int c[3];
         double f[3];
-        long long w[3][2];
         locate(g, x, c, f);
-        qweights(f, w);
+        const Cic w(f);
         const double cell = (double)cell_of(g, c);
         pos_e[se] = make_double4(x[0], x[1], x[2], cell);
         vel_e[se] = make_double4(cr.ve[0], cr.ve[1], cr.ve[2], (double)(nid + (unsigned)(2 * rank)));
         pos_i[si] = make_double4(x[0], x[1], x[2], cell);
         vel_i[si] = make_double4(cr.vi[0], cr.vi[1], cr.vi[2], (double)(nid + (unsigned)(2 * rank + 1)));
-        deposit(g, rq, c, w, -1);
-        deposit(g, rq, c, w, 1);
+        deposit(g, rq, c, w.a, -1);
+        deposit(g, rq, c, w.a, 1);
     }
 }
 
@@ -549,10 +719,15 @@ __global__ void k_grains(Geo g, int ng, double qw, const unsigned long long* gab
     const double x[3] = {gpos[3 * gi], gpos[3 * gi + 1], gpos[3 * gi + 2]};
     int c[3];
     double f[3];
-    long long w[3][2];
     locate(g, x, c, f);
-    qweights(f, w);
-    deposit(g, rq, c, w, net);
+    const Cic w(f);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) {
+        const int di = d & 1, dy = (d >> 1) & 1, dz = d >> 2;
+        const long long v = net * ((long long)(di ? w.a[0] : kWQ - w.a[0]) * ((dy ? w.a[1] : kWQ - w.a[1]) *
+                                                                            (dz ? w.a[2] : kWQ - w.a[2])));
+        if (v != 0) atomicAdd(rq + corner(g, c, di, dy, dz), (unsigned long long)v);
+    }
 }
 
 // E of the current phi on the 4x4x4 nodes of grain gi's region (unit-charge table)
@@ -695,9 +870,9 @@ __global__ void k_grain_table_sup(Geo g, const double* gpos, const int* gcell, c
     const double x[3] = {gpos[3 * gi], gpos[3 * gi + 1], gpos[3 * gi + 2]};
     int c[3];
     double f[3];
-    long long w[3][2];
     locate(g, x, c, f);
-    qweights(f, w);
+    const Cic cic(f);
+    const long long w[3][2] = {{kWQ - cic.a[0], cic.a[0]}, {kWQ - cic.a[1], cic.a[1]}, {kWQ - cic.a[2], cic.a[2]}};
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int li = t % 4, lj = (t / 4) % 4, lk = t / 16;
     const int i = ((gcell[3 * gi] - 1 + li) % nx + nx) % nx;
@@ -733,15 +908,14 @@ __global__ void k_moments64(Geo g, const double4* pos, const double4* vel, const
         const double x[3] = {P.x, P.y, P.z};
         int c[3];
         double f[3];
-        long long w[3][2];
         locate(g, x, c, f);
-        qweights(f, w);
+        const Cic w(f);
         for (int dz = 0; dz < 2; ++dz)
             for (int dy = 0; dy < 2; ++dy)
                 for (int di = 0; di < 2; ++di) {
-                    const double wt = (double)(w[0][di] * w[1][dy] * w[2][dz]) * 0x1p-42;
+                    const double wt = w.w[0][di] * (w.w[1][dy] * w.w[2][dz]);
                     if (wt == 0.0) continue;
-                    const size_t node = node_at(g, c[0] + di, c[1] + dy, c[2] + dz);
+                    const size_t node = corner(g, c, di, dy, dz);
                     double* m = mom + 4 * node;
                     atomicAdd(m, wt);
                     atomicAdd(m + 1, wt * V.x);
@@ -752,7 +926,22 @@ __global__ void k_moments64(Geo g, const double4* pos, const double4* vel, const
     }
 }
 
-Geo geo(const pic_ctx* c) { return Geo{c->nx, c->ny, c->nz, c->dx, c->Lx, c->Ly, c->Lz}; }
+// (the reciprocal's corrections keep clear of under- and overflow in this range of dx)
+Geo geo(const pic_ctx* c)
+{
+    Geo g{c->nx, c->ny, c->nz, c->dx, c->Lx, c->Ly, c->Lz, 0.0, 0ull, 0};
+    if (c->dx > 1e-100 && c->dx < 1e100) {
+        g.rdx = 1.0 / c->dx;
+        // dx = D 2^(e - 53), 2^52 <= D < 2^53: 1 / dx = (2^116 / D) 2^(-63 - e)
+        int e = 0;
+        const unsigned long long D = (unsigned long long)std::ldexp(std::frexp(c->dx, &e), 53);
+        if (D == 1ull << 52) --e;
+        g.fix_c = D == 1ull << 52 ? 1ull << 63 : (unsigned long long)((((unsigned __int128)1) << 116) / D);
+        g.fix_e = e;
+        if (c->nx >= 65536 || c->ny >= 65536 || c->nz >= 65536) g.fix_c = 0ull;
+    }
+    return g;
+}
 
 
 // Initial plasma drawn from the run's seed, the same definition the oracle
@@ -893,7 +1082,7 @@ void launch_stage_particles(pic_ctx* c, int sp, const double* x, const double* v
 {
     if (n <= 0) return;
     StageP p;
-    p.g = Geo{c->nx, c->ny, c->nz, c->dx, c->Lx, c->Ly, c->Lz};
+    p.g = geo(c);
     p.vs = c->dt / c->dx;
     p.x = x;
     p.v = v;
@@ -913,18 +1102,22 @@ void launch_stage_particles(pic_ctx* c, int sp, const double* x, const double* v
 
 void launch_push64(pic_ctx* c)
 {
+    P64 ps[2];
     for (int sp = 0; sp < 2; ++sp) {
-        P64 p;
-        p.nx = c->nx; p.ny = c->ny; p.nz = c->nz;
-        p.dx = c->dx; p.Lx = c->Lx; p.Ly = c->Ly; p.Lz = c->Lz;
+        P64& p = ps[sp];
+        p.g = geo(c);
+        p.Lx = c->Lx; p.Ly = c->Ly;
         p.M = c->md_sub > 0 ? c->md_sub : 1;
         p.dt = c->dt;
         p.dtm = c->dt / (double)p.M;
         p.sp = sp;
-        p.qmdt = c->qm[sp] * c->dt;
+        p.qmdt = (c->qm[sp] * c->dt) * 0x1p-42;   // for gather_scaled
         p.qmdtm = c->qm[sp] * p.dtm;
         p.hm = c->hm[sp];
-        p.pnull = c->pnull[sp];
+        const double below = std::ceil(c->pnull[sp] * 0x1p32 - 0.5);   // u + 1/2 < pnull 2^32
+        p.null_below = below > 0.0 ? (unsigned long long)below : 0ull;
+        p.mcc_list = c->mcc_list[sp];
+        p.mcc_n = c->d_lists + 2 * sp + 1;
         p.nu_max = c->nu_max[sp];
         p.de = c->de[sp];
         p.n_gas = c->n_gas;
@@ -951,7 +1144,13 @@ void launch_push64(pic_ctx* c)
         p.child = c->d_child;
         p.child_cap = (unsigned long long)c->child_cap;
         p.nch = c->d_nch;
-        k_push64<<<grid_for(c->cap[sp], 128, 152 * 16), 128, 0, c->stream>>>(p);
+    }
+    cudaMemsetAsync(c->d_lists, 0, 4 * sizeof(unsigned int), c->stream);
+    const int64_t most = std::max(c->cap[0], c->cap[1]);
+    k_push64<<<dim3((unsigned)grid_for(most, kPush64Threads, 152 * 16), 2), kPush64Threads, 0, c->stream>>>(ps[0], ps[1]);
+    c->launches += 1;
+    if (!(c->flags & PIC_F_NO_MCC)) {
+        k_mcc64<<<dim3(152 * 4, 2), kPush64Threads, 0, c->stream>>>(ps[0], ps[1]);
         c->launches += 1;
     }
 }
@@ -1024,7 +1223,7 @@ void launch_init_plasma(pic_ctx* c, int sp, int64_t n, uint32_t id0, double t_ev
 {
     if (n <= 0) return;
     InitP p;
-    p.g = Geo{c->nx, c->ny, c->nz, c->dx, c->Lx, c->Ly, c->Lz};
+    p.g = geo(c);
     p.key = c->key;
     p.n = n;
     p.id0 = id0;
