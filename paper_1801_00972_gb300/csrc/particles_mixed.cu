@@ -261,18 +261,6 @@ __device__ __forceinline__ int carry(int nx, int ny, int nz, int& i, int& j, int
     return 0;
 }
 
-// separation from grain gi in cell units, minimum image in x and y
-__device__ __forceinline__ void grain_sep(const P32& p, int gi, int i, int j, int k, const float o[3], float d[3])
-{
-    int di = i - p.gcell[3 * gi], dj = j - p.gcell[3 * gi + 1];
-    const int dk = k - p.gcell[3 * gi + 2];
-    if (di > p.nx / 2) di -= p.nx; else if (di < -p.nx / 2) di += p.nx;
-    if (dj > p.ny / 2) dj -= p.ny; else if (dj < -p.ny / 2) dj += p.ny;
-    d[0] = (float)di + (o[0] - p.goff[3 * gi]);
-    d[1] = (float)dj + (o[1] - p.goff[3 * gi + 1]);
-    d[2] = (float)dk + (o[2] - p.goff[3 * gi + 2]);
-}
-
 __device__ __forceinline__ float xs_at(const float* tab, int n, float de, float eps)
 {
     const float t = eps / de;
@@ -627,16 +615,31 @@ __global__ void k_tile_md(int ng, const int* gcell, int nx, int ny, int nz, int 
     }
 }
 
+constexpr int kMdLanes = 4;
+constexpr int kMdThreads = 64;
+
 // Field data of one cell for the MD substeps: the 8 corner values of
-// E_PIC - sum_g Q_g g_g (Eq. 5, mesh part) and the cell's near grains, so a
-// substep that stays in its cell touches no memory.
+// E_PIC - sum_g Q_g g_g (Eq. 5, mesh part) in registers and the cell's near
+// grains in the thread's column of shared memory, so a substep that stays in its
+// cell touches no global memory.
 struct MdCell {
     float ec[8][3];
     int ng;
-    int gi[kMaxG];
+};
+struct MdGrains {
+    // per grain: its cell seen from the particle's (minimum image in x and y), its
+    // offset inside its cell, Q / (4 pi eps0 dx^2), (radius / dx)^2, index
+    float v[kMaxG][8][kMdThreads];
+    int gi[kMaxG][kMdThreads];
+    // separation of offsets o in the particle's cell from grain t, in cell units
+    __device__ __forceinline__ void sep(int t, const float o[3], float d[3]) const
+    {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) d[a] = v[t][a][threadIdx.x] + (o[a] - v[t][3 + a][threadIdx.x]);
+    }
 };
 
-__device__ void md_load(const P32& p, int i, int j, int k, MdCell& m)
+__device__ void md_load(const P32& p, int i, int j, int k, MdCell& m, MdGrains& mg)
 {
     const int i1 = (i + 1 == p.nx) ? 0 : i + 1;
     const int j1 = (j + 1 == p.ny) ? 0 : j + 1;
@@ -650,9 +653,16 @@ __device__ void md_load(const P32& p, int i, int j, int k, MdCell& m)
     m.ng = p.cell_ng[cell];
     for (int t = 0; t < m.ng; ++t) {
         const int gi = p.cell_g[cell * kMaxG + t];
-        m.gi[t] = gi;
         const float Q = p.gq[gi];
         const int gc0 = p.gcell[3 * gi], gc1 = p.gcell[3 * gi + 1], gc2 = p.gcell[3 * gi + 2];
+        int di = i - gc0, dj = j - gc1;
+        if (di > p.nx / 2) di -= p.nx; else if (di < -p.nx / 2) di += p.nx;
+        if (dj > p.ny / 2) dj -= p.ny; else if (dj < -p.ny / 2) dj += p.ny;
+        const float g[8] = {(float)di, (float)dj, (float)(k - gc2), p.goff[3 * gi], p.goff[3 * gi + 1], p.goff[3 * gi + 2],
+                            Q * p.qk, p.gr2[gi]};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) mg.v[t][c][threadIdx.x] = g[c];
+        mg.gi[t][threadIdx.x] = gi;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int li = ((i + (c & 1) - gc0 + 1) % p.nx + p.nx) % p.nx;
@@ -670,14 +680,27 @@ __device__ void md_load(const P32& p, int i, int j, int k, MdCell& m)
 // absorption after each substep, then MCC and the deposit (Sec. III).  Runs
 // beside k_push32, so the new states go to md_res and reach pos/vel only in
 // k_md_commit, after both have finished (k_push32 reads these slots' cells).
-__global__ void __launch_bounds__(64) k_md32(const P32 p)
+// A chain of md_sub dependent substeps per particle, so latency bound; a lane
+// that crosses into another cell holds its whole warp up for the new cell's
+// tables.  While the particles are few for the chip, a warp therefore takes
+// only kMdLanes of them, and both species (blockIdx.y) run side by side; the
+// grains near a cell lie in shared memory, not behind four levels of indices.
+// Particle phase of the 32 x 32 x 64-cell run with one grain: two launches, one
+// species after the other, 90 us; one launch, 32 lanes 64, 4 lanes 56 (8: 58, 1:
+// 56), with the grains in shared memory 52 us.
+__global__ void __launch_bounds__(kMdThreads) k_md32(const P32 pe, const P32 pi)
 {
+    __shared__ MdGrains mg;
+    const P32& p = blockIdx.y == 0 ? pe : pi;
     if (p.sp == 1 && (p.flags & PIC_F_IONS_FROZEN)) return;
     const unsigned int n = *p.md_n;
+    const unsigned int warps = gridDim.x * (kMdThreads / 32), lane = threadIdx.x & 31u;
+    const unsigned int per = n <= warps * kMdLanes ? (unsigned int)kMdLanes : 32u;   // particles per warp
+    if (lane >= per) return;
     const uint32_t step = *p.step;
     const long long charge = p.sp == 0 ? -1 : 1;
     const float s = 1.0f / (float)kWQ;
-    for (unsigned int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
+    for (unsigned int t = (blockIdx.x * (kMdThreads / 32) + (threadIdx.x >> 5)) * per + lane; t < n; t += warps * per) {
         const unsigned int q = p.md_list[t];
         const float4 P = p.pos[q];
         const float4 V = p.vel[q];
@@ -691,7 +714,7 @@ __global__ void __launch_bounds__(64) k_md32(const P32 p)
         float v[3] = {V.x, V.y, V.z};
         int fate = 0, grain = -1;
         MdCell mc;
-        md_load(p, i, j, k, mc);
+        md_load(p, i, j, k, mc, mg);
         for (int m = 0; m < p.M; ++m) {
             const int a0 = qa(o[0]), a1 = qa(o[1]), a2 = qa(o[2]);
             const float wx[2] = {(float)(kWQ - a0) * s, (float)a0 * s};
@@ -707,21 +730,21 @@ __global__ void __launch_bounds__(64) k_md32(const P32 p)
             }
             for (int g = 0; g < mc.ng; ++g) {      // Eq. 6: Coulomb field of the near grains
                 float d[3];
-                grain_sep(p, mc.gi[g], i, j, k, o, d);
+                mg.sep(g, o, d);
                 const float r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                const float coef = r2 > 0.f ? (p.gq[mc.gi[g]] * p.qk) / (r2 * sqrtf(r2)) : 0.f;
+                const float coef = r2 > 0.f ? mg.v[g][6][threadIdx.x] / (r2 * sqrtf(r2)) : 0.f;
                 E[0] += coef * d[0]; E[1] += coef * d[1]; E[2] += coef * d[2];
             }
             v[0] += E[0] * p.kqm; v[1] += E[1] * p.kqm; v[2] += E[2] * p.kqm;
             o[0] += v[0] * p.invM; o[1] += v[1] * p.invM; o[2] += v[2] * p.invM;
-            const int pi = i, pj = j, pk = k;
+            const int ci = i, cj = j, ck = k;
             fate = carry(p.nx, p.ny, p.nz, i, j, k, o);
             if (fate) break;
-            if (i != pi || j != pj || k != pk) md_load(p, i, j, k, mc);
+            if (i != ci || j != cj || k != ck) md_load(p, i, j, k, mc, mg);
             for (int g = 0; g < mc.ng && grain < 0; ++g) {
                 float d[3];
-                grain_sep(p, mc.gi[g], i, j, k, o, d);
-                if (d[0] * d[0] + d[1] * d[1] + d[2] * d[2] <= p.gr2[mc.gi[g]]) grain = mc.gi[g];
+                mg.sep(g, o, d);
+                if (d[0] * d[0] + d[1] * d[1] + d[2] * d[2] <= mg.v[g][7][threadIdx.x]) grain = mg.gi[g][threadIdx.x];
             }
             if (grain >= 0) break;
         }
@@ -1076,8 +1099,7 @@ void launch_push32(pic_ctx* c)
     const P32 pe = params(c, 0), pi = params(c, 1);
     cudaEventRecord(c->ev_fork, c->stream);
     cudaStreamWaitEvent(c->aux, c->ev_fork, 0);
-    k_md32<<<152 * 4, 64, 0, c->aux>>>(pe);
-    k_md32<<<152 * 4, 64, 0, c->aux>>>(pi);
+    k_md32<<<dim3(152 * 8, 2), kMdThreads, 0, c->aux>>>(pe, pi);
     cudaEventRecord(c->ev_join, c->aux);
     // both species of a tile in one block: one window, one flush
     const unsigned grid = (unsigned)(c->ntiles + kTailBlocks);
@@ -1095,7 +1117,7 @@ void launch_push32(pic_ctx* c)
                                            (float4*)c->pos[1], (float4*)c->vel[1], c->md_list[1], c->md_res[1],
                                            c->d_lists, (unsigned int)c->md_rescap,
                                            (c->flags & PIC_F_IONS_FROZEN) ? 1 : 0);
-    c->launches += 8;
+    c->launches += 7;
 }
 
 // The attribute belongs to the kernel, not to a run: it is raised to the
