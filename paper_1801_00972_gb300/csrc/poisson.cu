@@ -224,7 +224,15 @@ template <typename T> struct Two;
 template <> struct Two<float> { using V = float2; };
 template <> struct Two<double> { using V = double2; };
 
-template <typename T>
+// FROMF: the black half-sweep that follows a red one from a zero guess, the red
+// values formed on the way as that sweep would have (h^2 f / 6, rounded after
+// each product): the red half-sweep itself is left out, since the next one
+// computes every red node anew (256 x 256 x 1024 cells: 45 us less per
+// iteration; one launch less on every mesh).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+template <typename T, bool FROMF>
 __global__ void k_rbgs_split2(T* __restrict__ u, const T* __restrict__ f, Dims d, T h2, int color, int zero, int zp)
 {
     using V = typename Two<T>::V;
@@ -237,7 +245,7 @@ __global__ void k_rbgs_split2(T* __restrict__ u, const T* __restrict__ f, Dims d
     if (q >= qx || j >= d.ny || k0 >= k1) return;
     T* uc = u + (color ? d.half : 0);
     const T* fc = f + (color ? d.half : 0);
-    const T* uo = u + (color ? 0 : d.half);
+    const T* uo = (FROMF ? f : u) + (color ? 0 : d.half);
     int m = k0 * P2 + j * hx + 2 * q;   // even: 2-element aligned
     if (zero) {
         for (int k = k0; k < k1; ++k, m += P2) {
@@ -252,12 +260,18 @@ __global__ void k_rbgs_split2(T* __restrict__ u, const T* __restrict__ f, Dims d
     const int dl = (q == 0) ? hx - 1 : -1;            // pair 2q - 1
     const int dr = (q + 1 == qx) ? 2 - hx : 2;        // pair 2q + 2
     const int dyp = (j + 1 == d.ny) ? -j * hx : hx, dym = (j == 0) ? (d.ny - 1) * hx : -hx;
-    auto ld = [&](int at) { return *reinterpret_cast<const V*>(uo + at); };
+    auto one = [&](T v) { return FROMF ? mul_rn(mul_rn(h2, v), (T)(1.0 / 6.0)) : v; };
+    auto ld = [&](int at) {
+        V v = *reinterpret_cast<const V*>(uo + at);
+        v.x = one(v.x);
+        v.y = one(v.y);
+        return v;
+    };
     V om = ld(m - P2), oc = ld(m), op = ld(m + P2);
     for (int k = k0; k < k1; ++k, m += P2) {
         const V on = (k + 1 < k1) ? ld(m + 2 * P2) : op;
         const int p = (j + k + color) & 1;
-        const T ox = uo[m + (p ? dr : dl)];
+        const T ox = one(uo[m + (p ? dr : dl)]);
         const V yp = ld(m + dyp), ym = ld(m + dym);
         const V ff = *reinterpret_cast<const V*>(fc + m);
         const T xp0 = p ? oc.y : oc.x, xm0 = p ? oc.x : ox;
@@ -364,8 +378,9 @@ __global__ void k_resid_restrict(const T* __restrict__ u, const T* __restrict__ 
          res_at(u, f, df, i0, jm, k0 + 1, inv_h2) + res_at(u, f, df, i0, jp, k0 + 1, inv_h2);
     const T v = (T)0.125 * res_at(u, f, df, i0, j0, k0, inv_h2) + (T)0.03125 * e;
     const int nc = K * dc.nx * dc.ny + J * dc.nx + I;
-    fc[nc] = v;
-    if (((I + J + K) & 1) == 0) uc[nc] = h2c * v * (T)(1.0 / 6.0);
+    const int col = (I + J + K) & 1;
+    fc[lix(dc, nc, col)] = v;
+    if (col == 0) uc[lix(dc, nc, 0)] = h2c * v * (T)(1.0 / 6.0);
 }
 
 // trilinear interpolation of the coarse correction, added on the fine interior
@@ -536,10 +551,13 @@ __global__ void k_restrict_red(const T* __restrict__ rr, T* __restrict__ fc, T* 
     if (col == 0) uc[lix(dc, nc, 0)] = h2c * v * (T)(1.0 / 6.0);
 }
 
-// k_prolong_cell onto a split level: thread (I, J) walks zp coarse
-// planes of its column, the corners of plane K + 1 reused as those of the
-// next cell's plane K; the fine pair (I, 2J + b, 2K + c) gets its two nodes'
-// values added at pair index m in the red and black halves.
+// k_prolong_cell onto a split level, black nodes only: the red half-sweep that
+// starts the post-smoothing computes every red node anew from its black
+// neighbours (omega = 1), so what the prolongation would add there is never
+// read.  Thread (I, J) walks zp coarse planes of its column, the corners of plane
+// K + 1 reused as those of the next cell's plane K; of the fine pair (I, 2J + b,
+// 2K + c) node 0 is black where b + c is odd, else node 1.  Fine level of 256 x
+// 256 x 1024 cells: 88 us for both colours, 45 for the black.
 template <typename T>
 __global__ void k_prolong_split(T* __restrict__ uf, const T* __restrict__ uc, Dims df, Dims dc, int zp)
 {
@@ -551,28 +569,23 @@ __global__ void k_prolong_split(T* __restrict__ uf, const T* __restrict__ uc, Di
     if (I >= dc.nx || J >= dc.ny || Kb >= Ke) return;
     const int I1 = (I + 1 == dc.nx) ? 0 : I + 1, J1 = (J + 1 == dc.ny) ? 0 : J + 1;
     const int Pc = dc.nx * dc.ny, hx = df.nx >> 1, P2 = hx * df.ny;
+    T* ub = uf + df.half;
     // a corner of coarse plane K (the coarse level may itself be split)
     auto cr = [&](int K, int i, int j) { return uc[lix(dc, K * Pc + j * dc.nx + i, (i + j + K) & 1)]; };
     T c000 = cr(Kb, I, J), c001 = cr(Kb, I1, J), c010 = cr(Kb, I, J1), c011 = cr(Kb, I1, J1);
     for (int K = Kb; K < Ke; ++K) {
         const T c100 = cr(K + 1, I, J), c101 = cr(K + 1, I1, J), c110 = cr(K + 1, I, J1), c111 = cr(K + 1, I1, J1);
-        // the 8 fine values of this cell: addresses and old values first (all
-        // loads in flight together), then the sums and stores
-        int adr[2][2][2];
-        T old[2][2][2];
+        // the 4 black fine values of this cell: old values first (all loads in
+        // flight together), then the sums and stores
+        const int m0 = (2 * K) * P2 + (2 * J) * hx + I;
+        const int adr[2][2] = {{m0, m0 + hx}, {m0 + P2, m0 + P2 + hx}};
+        T old[2][2];
 #pragma unroll
-        for (int cz = 0; cz < 2; ++cz)
+        for (int cz = 0; cz < 2; ++cz) {
+            const bool in = 2 * K + cz >= 1 && 2 * K + cz <= df.nz - 1;
 #pragma unroll
-            for (int by = 0; by < 2; ++by) {
-                const int k = 2 * K + cz, j = 2 * J + by;
-                const int m = k * P2 + j * hx + I;
-                const int c0 = (j + k) & 1;   // colour of node 0 of the pair
-                adr[cz][by][0] = (c0 ? df.half : 0) + m;
-                adr[cz][by][1] = (c0 ? 0 : df.half) + m;
-                const bool in = k >= 1 && k <= df.nz - 1;
-#pragma unroll
-                for (int bx = 0; bx < 2; ++bx) old[cz][by][bx] = in ? uf[adr[cz][by][bx]] : (T)0;
-            }
+            for (int by = 0; by < 2; ++by) old[cz][by] = in ? ub[adr[cz][by]] : (T)0;
+        }
 #pragma unroll
         for (int cz = 0; cz < 2; ++cz) {
             const int k = 2 * K + cz;
@@ -580,14 +593,13 @@ __global__ void k_prolong_split(T* __restrict__ uf, const T* __restrict__ uc, Di
             const T z0[4] = {c000, c001, c010, c011};
             const T z1[4] = {cz ? c100 : c000, cz ? c101 : c001, cz ? c110 : c010, cz ? c111 : c011};
 #pragma unroll
-            for (int by = 0; by < 2; ++by)
-#pragma unroll
-                for (int bx = 0; bx < 2; ++bx) {
-                    const T p00 = z0[0], p01 = z0[bx ? 1 : 0], p10 = z0[by ? 2 : 0], p11 = z0[(by ? 2 : 0) + (bx ? 1 : 0)];
-                    const T q00 = z1[0], q01 = z1[bx ? 1 : 0], q10 = z1[by ? 2 : 0], q11 = z1[(by ? 2 : 0) + (bx ? 1 : 0)];
-                    const T v = (T)0.125 * (p00 + p01 + p10 + p11 + q00 + q01 + q10 + q11);
-                    uf[adr[cz][by][bx]] = old[cz][by][bx] + v;
-                }
+            for (int by = 0; by < 2; ++by) {
+                const int bx = (by + cz) & 1 ? 0 : 1;
+                const T p00 = z0[0], p01 = z0[bx ? 1 : 0], p10 = z0[by ? 2 : 0], p11 = z0[(by ? 2 : 0) + (bx ? 1 : 0)];
+                const T q00 = z1[0], q01 = z1[bx ? 1 : 0], q10 = z1[by ? 2 : 0], q11 = z1[(by ? 2 : 0) + (bx ? 1 : 0)];
+                const T v = (T)0.125 * (p00 + p01 + p10 + p11 + q00 + q01 + q10 + q11);
+                ub[adr[cz][by]] = old[cz][by] + v;
+            }
         }
         c000 = c100;
         c001 = c101;
@@ -1284,34 +1296,73 @@ __device__ __forceinline__ void st4(double* p, const double v[4])
 // Out[r][c] = scale * sum_s X(r, s) Y(s, c) on one 4 x 4 tile, with X read
 // as four rows (one value each per s, rows xp apart) or as a 4-vector per s,
 // and Y as a 4-vector per s.
-template <typename T, bool XVEC>
-__device__ __forceinline__ void tile4(const T* x, int xs, int xp, const T* y, int ys, int n, T acc[4][4])
+template <typename T, bool XVEC, int RA>
+__device__ __forceinline__ void tile4(const T* x, int xs, int xp, const T* y, int ys, int n, T acc[RA][4])
 {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RA; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
 #pragma unroll 4
     for (int s = 0; s < n; ++s) {
         T xv[4], yv[4];
-        if (XVEC) {
+        if (XVEC && RA == 4) {
             ld4(x + s * xs, xv);
         } else {
 #pragma unroll
-            for (int a = 0; a < 4; ++a) xv[a] = x[a * xp + s * xs];
+            for (int a = 0; a < RA; ++a) xv[a] = x[a * xp + s * xs];
         }
         ld4(y + s * ys, yv);
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < RA; ++a)
 #pragma unroll
             for (int b = 0; b < 4; ++b) acc[a][b] += xv[a] * yv[b];
     }
 }
 
+// The four transforms of a CTA's nk planes, RA x 4 values per thread (each
+// value's sum in the same order for any RA).
+//   rows: O[row][c] = sum_s X[row][s] Y[s][c]
+template <typename T, int RA, typename OUT>
+__device__ __forceinline__ void exact_rows(const T* X, int rp, int rows, const T* Y, int n, FastDiv f_n4, OUT out)
+{
+    const int n4 = n / 4;
+    for (int q = threadIdx.x; q < rows / RA * n4; q += blockDim.x) {
+        const int rg = fdiv(q, f_n4), cg4 = q - rg * n4;
+        T acc[RA][4];
+        tile4<T, false, RA>(X + RA * rg * rp, 1, rp, Y + 4 * cg4, n, n, acc);
+#pragma unroll
+        for (int a = 0; a < RA; ++a) out(RA * rg + a, 4 * cg4, acc[a]);
+    }
+}
+//   columns: O[plane][r][c] = sum_s Qt[s][r] X[plane][s][c] (times `scale` where asked)
+template <typename T, int RA, bool SCALE>
+__device__ __forceinline__ void exact_cols(const T* Qt, const T* X, T* O, int nk, int ny, int nx, int rp, int pp,
+                                           const FastDiv& f_t, const FastDiv& f_x4, T scale)
+{
+    const int nx4 = nx / 4, per = ny / RA * nx4;
+    for (int q = threadIdx.x; q < nk * per; q += blockDim.x) {
+        const int kk = RA == 4 ? fdiv(q, f_t) : q / per, rem = q - kk * per;
+        const int rg = fdiv(rem, f_x4), cg4 = rem - rg * nx4;
+        T acc[RA][4];
+        tile4<T, true, RA>(Qt + RA * rg, ny, 1, X + kk * pp + 4 * cg4, rp, ny, acc);
+#pragma unroll
+        for (int a = 0; a < RA; ++a) {
+            if (SCALE)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) acc[a][b] *= scale;
+            st4(O + kk * pp + (RA * rg + a) * rp + 4 * cg4, acc[a]);
+        }
+    }
+}
+
+// Latency bound (16 SMs, a few thousand values per phase): the constant tables
+// load before the wait for the right-hand side, few values go 4 per thread, the
+// z recurrences read ahead in registers.  By itself (ncu) 11.5 -> 10.2 us on
+// 16 x 16 x 32 cells, 14.9 -> 13.7 us on 16 x 16 x 64.
 template <typename T>
 __global__ void __launch_bounds__(kClThreads) k_coarse_exact(const ExactLevel<T> E)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     extern __shared__ __align__(16) unsigned char smem[];
     cg::cluster_group cl = cg::this_cluster();
     const int r = (int)cl.block_rank(), C = (int)cl.num_blocks();
@@ -1331,36 +1382,25 @@ __global__ void __launch_bounds__(kClThreads) k_coarse_exact(const ExactLevel<T>
     const int base = (klo - k0) * pp;   // first interior plane in A and B
     const int m0 = r * E.mm, nm = max(0, min(P, m0 + E.mm) - m0);
     const int nx4 = nx / 4;
+    // the constants before the wait for the level's right-hand side
     for (int q = t; q < 2 * nx * nx + 2 * ny * ny; q += bd) Qx[q] = E.Q[q];
+    for (int q = t; q < nm * N; q += bd) Pv[q] = E.p[(size_t)m0 * N + q];
+    pdl_begin();
     for (int q = t; q < nk * P; q += bd) {
         const int row = fdiv(q, E.f_x);   // kk ny + j
         A[base + row * rp + (q - row * nx)] = E.gf[(size_t)klo * P + q];
     }
-    for (int q = t; q < nm * N; q += bd) Pv[q] = E.p[(size_t)m0 * N + q];
     __syncthreads();
-    const int rows4 = nk * ny / 4;   // 4-row groups over all planes (ny is a multiple of 4)
+    const int rows = nk * ny;                     // (ny is a multiple of 4)
+    const bool wide = rows * nx4 <= 2 * bd;       // few values: 4 per thread instead of 16
     // forward along x: B[row][mx] = sum_i A[row][i] Qx[mx][i]
-    for (int q = t; q < rows4 * nx4; q += bd) {
-        const int rg = fdiv(q, E.f_x4), cg4 = q - rg * nx4;
-        T acc[4][4];
-        tile4<T, false>(A + base + 4 * rg * rp, 1, rp, QxT + 4 * cg4, nx, nx, acc);
-#pragma unroll
-        for (int a = 0; a < 4; ++a) st4(B + base + (4 * rg + a) * rp + 4 * cg4, acc[a]);
-    }
+    auto to_b = [&](int row, int c, const T (&v)[4]) { st4(B + base + row * rp + c, v); };
+    if (wide) exact_rows<T, 1>(A + base, rp, rows, QxT, nx, E.f_x4, to_b);
+    else exact_rows<T, 4>(A + base, rp, rows, QxT, nx, E.f_x4, to_b);
     __syncthreads();
     // forward along y, times h^2: A[my][mx] = h^2 sum_j Qy[my][j] B[j][mx]
-    for (int q = t; q < nk * (ny / 4) * nx4; q += bd) {
-        const int kk = fdiv(q, E.f_t2), rem = q - kk * (ny / 4) * nx4;
-        const int mg = fdiv(rem, E.f_x4), cg4 = rem - mg * nx4;
-        T acc[4][4];
-        tile4<T, true>(QyT + 4 * mg, ny, 0, B + base + kk * pp + 4 * cg4, rp, ny, acc);
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] *= E.h2;
-            st4(A + base + kk * pp + (4 * mg + a) * rp + 4 * cg4, acc[a]);
-        }
-    }
+    if (wide) exact_cols<T, 1, true>(QyT, B + base, A + base, nk, ny, nx, rp, pp, E.f_t2, E.f_x4, E.h2);
+    else exact_cols<T, 4, true>(QyT, B + base, A + base, nk, ny, nx, rp, pp, E.f_t2, E.f_x4, E.h2);
     cl.sync();
     // this CTA's modes: spectral right-hand sides from every plane's holder
     for (int q = t; q < nm * N; q += bd) {
@@ -1375,15 +1415,36 @@ __global__ void __launch_bounds__(kClThreads) k_coarse_exact(const ExactLevel<T>
     for (int mq = t; mq < nm; mq += bd) {
         T* g = G + mq * N;
         const T* pv = Pv + mq * N;
+        // eight values ahead in registers: the loads of a chunk do not wait for the
+        // stores of the one before
+        constexpr int W = 8;
         T acc = (T)0;
-        for (int k = 0; k < N; ++k) {
-            acc = (g[k] + acc) * pv[k];
-            g[k] = acc;
+        for (int k = 0; k < N; k += W) {
+            T a[W], p[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                a[u] = k + u < N ? g[k + u] : (T)0;
+                p[u] = k + u < N ? pv[k + u] : (T)0;
+            }
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                acc = (a[u] + acc) * p[u];
+                if (k + u < N) g[k + u] = acc;
+            }
         }
         T x = (T)0;
-        for (int k = N - 1; k >= 0; --k) {
-            x = g[k] + pv[k] * x;
-            g[k] = x;
+        for (int k = N - 1; k >= 0; k -= W) {
+            T a[W], p[W];
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                a[u] = k - u >= 0 ? g[k - u] : (T)0;
+                p[u] = k - u >= 0 ? pv[k - u] : (T)0;
+            }
+#pragma unroll
+            for (int u = 0; u < W; ++u) {
+                x = a[u] + p[u] * x;
+                if (k - u >= 0) g[k - u] = x;
+            }
         }
     }
     __syncthreads();
@@ -1397,23 +1458,13 @@ __global__ void __launch_bounds__(kClThreads) k_coarse_exact(const ExactLevel<T>
     }
     cl.sync();
     // inverse along y: B[j][mx] = sum_my Qy[my][j] A[my][mx]
-    for (int q = t; q < nk * (ny / 4) * nx4; q += bd) {
-        const int kk = fdiv(q, E.f_t2), rem = q - kk * (ny / 4) * nx4;
-        const int jg = fdiv(rem, E.f_x4), cg4 = rem - jg * nx4;
-        T acc[4][4];
-        tile4<T, true>(Qy + 4 * jg, ny, 0, A + base + kk * pp + 4 * cg4, rp, ny, acc);
-#pragma unroll
-        for (int a = 0; a < 4; ++a) st4(B + base + kk * pp + (4 * jg + a) * rp + 4 * cg4, acc[a]);
-    }
+    if (wide) exact_cols<T, 1, false>(Qy, A + base, B + base, nk, ny, nx, rp, pp, E.f_t2, E.f_x4, (T)1);
+    else exact_cols<T, 4, false>(Qy, A + base, B + base, nk, ny, nx, rp, pp, E.f_t2, E.f_x4, (T)1);
     __syncthreads();
     // inverse along x: u[row][i] = sum_mx B[row][mx] Qx[mx][i]
-    for (int q = t; q < rows4 * nx4; q += bd) {
-        const int rg = fdiv(q, E.f_x4), cg4 = q - rg * nx4;
-        T acc[4][4];
-        tile4<T, false>(B + base + 4 * rg * rp, 1, rp, Qx + 4 * cg4, nx, nx, acc);
-#pragma unroll
-        for (int a = 0; a < 4; ++a) st4(E.gu + (size_t)klo * P + (size_t)(4 * rg + a) * nx + 4 * cg4, acc[a]);
-    }
+    auto to_u = [&](int row, int c, const T (&v)[4]) { st4(E.gu + (size_t)klo * P + (size_t)row * nx + c, v); };
+    if (wide) exact_rows<T, 1>(B + base, rp, rows, Qx, nx, E.f_x4, to_u);
+    else exact_rows<T, 4>(B + base, rp, rows, Qx, nx, E.f_x4, to_u);
 }
 
 // shared-memory layout of the exact solve of level l on C CTAs; false if it does not fit
@@ -1465,13 +1516,15 @@ cudaError_t launch_exact(cudaStream_t s, const ExactLevel<T>& E, int C, size_t s
     cfg.blockDim = dim3(kClThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)C;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = !query && PIC_PDL ? 2 : 1;
     if (query) {
         cudaError_t e = cudaFuncSetAttribute(k_coarse_exact<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kClSmemMax);
@@ -1500,15 +1553,19 @@ inline Grid3 grid_norm(int nx, int ny, int planes)
     return g;
 }
 
+// a split level whose half-sweeps take two pairs per thread
+inline bool pairs_of_pairs(const Dims& d) { return d.half > 0 && d.nx % 4 == 0 && d.half % 2 == 0; }
+
 template <typename T>
-void run_rbgs(cudaStream_t s, T* u, const T* f, Dims d, T h2, int color, int zero)
+void run_rbgs(cudaStream_t s, T* u, const T* f, Dims d, T h2, int color, int zero, bool from_f = false)
 {
     if (d.half) {
-        if (d.nx % 4 == 0 && d.half % 2 == 0) {
+        if (pairs_of_pairs(d)) {
             Grid3 g = grid3(d.nx / 4, d.ny, 1);
             const int zp = column_planes(g, d.nz - 1, kRbPlanes);
             g.grid.z = (unsigned)std::max(1, (d.nz - 1 + zp - 1) / zp);
-            launch_pdl(s, g.grid, g.block, k_rbgs_split2<T>, u, f, d, h2, color, zero, zp);
+            if (from_f) launch_pdl(s, g.grid, g.block, k_rbgs_split2<T, true>, u, f, d, h2, color, zero, zp);
+            else launch_pdl(s, g.grid, g.block, k_rbgs_split2<T, false>, u, f, d, h2, color, zero, zp);
             return;
         }
         Grid3 g = grid3(d.nx / 2, d.ny, 1);
@@ -1617,11 +1674,14 @@ T* vcycle(pic_ctx* c, int l)
     T* u = (T*)L.u;
     T* f = (T*)L.f;
     // pre-smoothing from a zero guess: the first red pass needs no neighbours
-    // (on the coarser levels the restriction above has already made it)
+    // (on the coarser levels the restriction above has already made it), and the
+    // first black one can form its values itself (float: memory bound; FP64 would
+    // pay twelve products per node for two)
+    const bool from_f = sizeof(T) == 4 && l == 0 && kPre > 1 && pairs_of_pairs(d);
     for (int s = 0; s < kPre; ++s)
         for (int color = 0; color < 2; ++color) {
-            if (s == 0 && color == 0 && l > 0) continue;
-            run_rbgs<T>(c->stream, u, f, d, h2, color, s == 0 && color == 0);
+            if (s == 0 && color == 0 && (l > 0 || from_f)) continue;
+            run_rbgs<T>(c->stream, u, f, d, h2, color, s == 0 && color == 0, from_f && s == 0);
             c->launches += 1;
         }
     MGLevel& C = c->mg[l + 1];
