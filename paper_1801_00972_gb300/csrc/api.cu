@@ -996,10 +996,11 @@ pic_status step_enqueue(pic_ctx* c, int32_t n_steps)
         if (c->eepf) c->eepf_steps += 1;
         c->step += 1;
         if (sort) {
-            std::swap(c->pos[0], c->pos_alt[0]);
-            std::swap(c->pos[1], c->pos_alt[1]);
-            std::swap(c->vel[0], c->vel_alt[0]);
-            std::swap(c->vel[1], c->vel_alt[1]);
+            for (int sp = 0; sp < 2; ++sp)
+                if (sort_swaps(c, sp)) {
+                    std::swap(c->pos[sp], c->pos_alt[sp]);
+                    std::swap(c->vel[sp], c->vel_alt[sp]);
+                }
             c->parity ^= 1;
         }
         r = launch_solve_graph(c);

@@ -333,6 +333,7 @@ void launch_moments_phi(pic_ctx* c);
 
 // sort.cu
 void sort_particles(pic_ctx* c, int sp);
+bool sort_swaps(const pic_ctx* c, int sp);            // whether a sort leaves the species in its other buffers
 void count_live(pic_ctx* c);                         // live records of both species into d_live
 void scan_cells(pic_ctx* c, unsigned int* data);   // exclusive scan of one value per cell, in place
 

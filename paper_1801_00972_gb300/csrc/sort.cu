@@ -2,7 +2,8 @@
 // dropping dead slots.  The FP64 path sorts by linear cell index; the mixed
 // path by tile (blocks of tile[0] x tile[1] x tile[2] cells, tile-major, the
 // cells of a tile row-major inside it), so that each tile's particles occupy
-// one contiguous slot range, which the push hands to one thread block.  The
+// one contiguous slot range, which the push hands to one thread block; the
+// electrons' order by cell is made in two passes (sort_swaps).  The
 // order of particles inside a cell is not fixed (atomic scatter); nothing in a
 // step depends on it: the deposit is an exact integer sum and the random
 // numbers are keyed on particle ids.
@@ -19,7 +20,8 @@ constexpr int kScanBlock = kScanThreads * kScanPer;
 
 // sort key geometry: tiles of tx x ty x tz cells, ntx x nty tiles per plane;
 // order: 0 one key per cell, 1 one key per tile (no order inside it), 2 one key
-// per block of 2 x 2 x 2 cells inside the tile
+// per block of 2 x 2 x 2 cells inside the tile, kByTile the tile index itself
+constexpr int kByTile = 3;
 struct KeyGeo {
     int tx, ty, tz, ntx, nty, order;
 };
@@ -34,6 +36,7 @@ __device__ __forceinline__ int key_of(const float4& p, const KeyGeo& g)
     const int i = c & 1023, j = (c >> 10) & 1023, k = c >> 20;
     const int ti = i / g.tx, tj = j / g.ty, tk = k / g.tz;
     const int tile = (tk * g.nty + tj) * g.ntx + ti;
+    if (g.order == kByTile) return tile;
     if (g.order == 1) return tile * (g.tx * g.ty * g.tz);
     if (g.order == 2) {
         const int bx = (g.tx + 1) >> 1, by = (g.ty + 1) >> 1;
@@ -205,18 +208,94 @@ __global__ void k_tile_ranges(const unsigned int* cursor, unsigned int* tstart, 
         tstart[t] = t == 0 ? 0u : cursor[t * per_tile - 1];
 }
 
-// exclusive scan of n values in place through the per-level scratch buffers
-void scan(pic_ctx* c, unsigned int* data, size_t n, int level)
+// The second pass of the electrons' sort: one block per tile puts the tile's
+// particles in cell order, from the buffers that the first pass sorted by tile
+// into the others, slot range for slot range.  Counts per cell in shared memory,
+// their exclusive scan, then each particle's place; up to kPermMax particles as
+// a permutation (reads scattered inside the tile's few ten KB, writes in whole
+// lines), more of them written to their places directly.
+constexpr int kOrderThreads = 256;
+constexpr int kOrderCells = 4096;   // largest tile, in cells
+constexpr int kPermMax = 8192;
+
+__global__ void __launch_bounds__(kOrderThreads) k_order_cells(const float4* __restrict__ pos, const float4* __restrict__ vel,
+                                                               const unsigned int* __restrict__ tstart,
+                                                               float4* __restrict__ pos_out, float4* __restrict__ vel_out,
+                                                               KeyGeo kg, int nx, int ny, const unsigned char* tile_md,
+                                                               const int* cell_ng, unsigned int* md_next, unsigned int* next_n)
+{
+    extern __shared__ unsigned int s_cell[];          // per cell: count, then next place
+    __shared__ unsigned int warp_tot[kOrderThreads / 32];
+    __shared__ unsigned short perm[kPermMax];
+    const unsigned int first = tstart[blockIdx.x], n = tstart[blockIdx.x + 1] - first;
+    if (n == 0u) return;
+    const int per = kg.tx * kg.ty * kg.tz, t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int k_first = (int)blockIdx.x * per;        // key of the tile's first cell
+    for (int q = t; q < per; q += kOrderThreads) s_cell[q] = 0u;
+    __syncthreads();
+    for (unsigned int q = t; q < n; q += kOrderThreads) atomicAdd(&s_cell[key_of(pos[first + q], kg) - k_first], 1u);
+    __syncthreads();
+    // exclusive scan: a run of cells per thread
+    const int each = (per + kOrderThreads - 1) / kOrderThreads, c0 = min(t * each, per), c1 = min(c0 + each, per);
+    unsigned int sum = 0u;
+    for (int q = c0; q < c1; ++q) sum += s_cell[q];
+    unsigned int incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned int y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+    }
+    if (lane == 31) warp_tot[w] = incl;
+    __syncthreads();
+    unsigned int run = incl - sum;
+    for (int q = 0; q < w; ++q) run += warp_tot[q];
+    for (int q = c0; q < c1; ++q) {
+        const unsigned int here = s_cell[q];
+        s_cell[q] = run;
+        run += here;
+    }
+    __syncthreads();
+    const bool md = md_next && tile_md[blockIdx.x];   // (the tile's own cells lie in its window)
+    auto list_md = [&](const float4& p, unsigned int slot) {
+        const int pc = __float_as_int(p.w);
+        if (cell_ng[((pc >> 20) * ny + ((pc >> 10) & 1023)) * nx + (pc & 1023)] != 0) md_next[atomicAdd(next_n, 1u)] = slot;
+    };
+    if (n <= kPermMax) {
+        for (unsigned int q = t; q < n; q += kOrderThreads)
+            perm[atomicAdd(&s_cell[key_of(pos[first + q], kg) - k_first], 1u)] = (unsigned short)q;
+        __syncthreads();
+#pragma unroll 4
+        for (unsigned int q = t; q < n; q += kOrderThreads) {
+            const unsigned int from = first + perm[q];
+            const float4 p = pos[from], v = vel[from];
+            pos_out[first + q] = p;
+            vel_out[first + q] = v;
+            if (md) list_md(p, first + q);
+        }
+    } else {
+        for (unsigned int q = t; q < n; q += kOrderThreads) {
+            const float4 p = pos[first + q], v = vel[first + q];
+            const unsigned int to = first + atomicAdd(&s_cell[key_of(p, kg) - k_first], 1u);
+            pos_out[to] = p;
+            vel_out[to] = v;
+            if (md) list_md(p, to);
+        }
+    }
+}
+
+// exclusive scan of n values in place through the per-level scratch buffers;
+// returns where the device finds their sum
+unsigned int* scan(pic_ctx* c, unsigned int* data, size_t n, int level)
 {
     const size_t nb = (n + kScanBlock - 1) / kScanBlock;
     unsigned int* sums = c->scan_tmp[level];
     k_scan_block<<<(unsigned)nb, kScanThreads, 0, c->stream>>>(data, data, sums, n);
     c->launches += 1;
-    if (nb > 1) {
-        scan(c, sums, nb, level + 1);
-        k_scan_add<<<grid_for((int64_t)n, 256, 152 * 8), 256, 0, c->stream>>>(data, sums, n);
-        c->launches += 1;
-    }
+    if (nb == 1) return sums;
+    unsigned int* total = scan(c, sums, nb, level + 1);
+    k_scan_add<<<grid_for((int64_t)n, 256, 152 * 8), 256, 0, c->stream>>>(data, sums, n);
+    c->launches += 1;
+    return total;
 }
 
 }  // namespace
@@ -257,38 +336,68 @@ void count_live(pic_ctx* c)
     c->launches += 2;
 }
 
+// Electrons in cell order take two passes: by tile, then by cell inside each
+// tile.  They cross about a third of a cell per step and axis, so a few steps after
+// a sort a tile's electrons are spread over three times its cells: a scatter
+// straight to cells is 32 separate 16-byte writes per warp and nearly one
+// returning atomic per particle.  Most of a warp goes to one or a few tiles,
+// though, and inside a tile the rest is local.  2.5e8 electrons on 256 x 256 x
+// 1024 cells, sorted every 5 steps: histogram 1.6 and scatter 14.8 ms in one
+// pass; 1.1, 3.0 and 3.7 ms in two (16 GB each of records read and written:
+// 2.6 ms is the memory's).  Ions hardly move between
+// sorts: their one pass writes whole lines already (3.4 ms).  Tiles of fewer than
+// 64 cells leave a block of the second pass too little to do, larger ones than
+// kOrderCells do not fit its counters; those take the one pass.
+bool sort_swaps(const pic_ctx* c, int sp)
+{
+    const bool two = c->prec == PIC_MIXED && sp == 0 && c->sort_order == 0 &&
+                     c->tile[0] * c->tile[1] * c->tile[2] >= kOrderThreads / 4 &&
+                     c->tile[0] * c->tile[1] * c->tile[2] <= kOrderCells;
+    return !two;
+}
+
 void sort_particles(pic_ctx* c, int sp)
 {
-    const size_t nk = c->nkeys;
-    const KeyGeo kg{c->tile[0], c->tile[1], c->tile[2], c->ntile[0], c->ntile[1], c->sort_order};
+    const bool mixed = c->prec == PIC_MIXED, two = !sort_swaps(c, sp);
+    const int per = c->tile[0] * c->tile[1] * c->tile[2];
+    const size_t nk = two ? (size_t)c->ntiles : c->nkeys;
+    KeyGeo kg{c->tile[0], c->tile[1], c->tile[2], c->ntile[0], c->ntile[1], two ? kByTile : c->sort_order};
     cudaMemsetAsync(c->cursor, 0, sizeof(unsigned int) * nk, c->stream);
     const int grid = grid_for(c->cap[sp], 256, 152 * 8);
-    if (c->prec == PIC_MIXED)
+    if (mixed)
         k_hist<float4><<<grid, 256, 0, c->stream>>>((const float4*)c->pos[sp], c->d_nslot, sp, c->cursor, kg);
     else
         k_hist<double4><<<grid, 256, 0, c->stream>>>((const double4*)c->pos[sp], c->d_nslot, sp, c->cursor, kg);
-    scan(c, c->cursor, nk, 0);
-    if (c->prec == PIC_MIXED) cudaMemsetAsync(c->d_lists + 4 + sp, 0, sizeof(unsigned int), c->stream);
-    if (c->prec == PIC_MIXED)
+    const unsigned int* total = scan(c, c->cursor, nk, 0);
+    if (mixed) cudaMemsetAsync(c->d_lists + 4 + sp, 0, sizeof(unsigned int), c->stream);
+    if (mixed)
         k_scatter<float4><<<grid, 256, 0, c->stream>>>((const float4*)c->pos[sp], (const float4*)c->vel[sp],
                                                        c->d_nslot, sp, c->cursor, (float4*)c->pos_alt[sp],
                                                        (float4*)c->vel_alt[sp], kg, c->nx, c->ny, c->cell_ng,
-                                                       c->md_next[sp], c->d_lists + 4 + sp);
+                                                       two ? nullptr : c->md_next[sp], c->d_lists + 4 + sp);
     else
         k_scatter<double4><<<grid, 256, 0, c->stream>>>((const double4*)c->pos[sp], (const double4*)c->vel[sp],
                                                         c->d_nslot, sp, c->cursor, (double4*)c->pos_alt[sp],
                                                         (double4*)c->vel_alt[sp], kg, c->nx, c->ny, c->cell_ng,
                                                         (unsigned int*)nullptr, (unsigned int*)nullptr);
     // the last scan level's single block sum is the number of live particles
-    k_set_nslot<<<1, 1, 0, c->stream>>>(c->d_nslot, sp, c->scan_tmp.back());
+    k_set_nslot<<<1, 1, 0, c->stream>>>(c->d_nslot, sp, total);
     c->launches += 3;
-    if (c->prec == PIC_MIXED) {
+    if (mixed) {
         k_tile_ranges<<<grid_for(c->ntiles + 1, 256, 152 * 4), 256, 0, c->stream>>>(
-            c->cursor, c->tstart[sp], (long long)c->ntiles, c->tile[0] * c->tile[1] * c->tile[2]);
+            c->cursor, c->tstart[sp], (long long)c->ntiles, two ? 1 : per);
         c->launches += 1;
     }
-    void* t = c->pos[sp]; c->pos[sp] = c->pos_alt[sp]; c->pos_alt[sp] = t;
-    t = c->vel[sp]; c->vel[sp] = c->vel_alt[sp]; c->vel_alt[sp] = t;
+    if (two) {
+        kg.order = 0;
+        k_order_cells<<<(unsigned)c->ntiles, kOrderThreads, sizeof(unsigned int) * (size_t)per, c->stream>>>(
+            (const float4*)c->pos_alt[sp], (const float4*)c->vel_alt[sp], c->tstart[sp], (float4*)c->pos[sp],
+            (float4*)c->vel[sp], kg, c->nx, c->ny, c->tile_md, c->cell_ng, c->md_next[sp], c->d_lists + 4 + sp);
+        c->launches += 1;
+        return;
+    }
+    std::swap(c->pos[sp], c->pos_alt[sp]);
+    std::swap(c->vel[sp], c->vel_alt[sp]);
 }
 
 }  // namespace pic
