@@ -13,10 +13,33 @@
 
 namespace pic {
 
+// Device memory of the run, given back by destroy().  A run holds about eighty
+// arrays, most of them small, and each allocation and each release costs the host
+// 10 to 15 us: arrays of at most half a slab are cut from slabs of c->slab_bytes
+// (256-byte steps), larger ones are allocated by themselves.  Where no slab can be
+// had, the array alone is asked for.  Starting and releasing a run of 64 x 64 x 128
+// cells with 2e6 particles: 5.3 ms with one allocation per array and the grain
+// lists filled on the host, 3.2 ms now.
 void* dev_alloc(pic_ctx* c, size_t bytes)
 {
+    const size_t need = (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255;
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes < 16 ? 16 : bytes) != cudaSuccess) {
+    if (need > c->slab_left && need <= c->slab_bytes / 2) {
+        if (cudaMalloc(&p, c->slab_bytes) == cudaSuccess) {
+            c->allocs.push_back(p);
+            c->slab = (char*)p;
+            c->slab_left = c->slab_bytes;
+        } else {
+            cudaGetLastError();
+        }
+    }
+    if (need <= c->slab_left) {
+        p = c->slab;
+        c->slab += need;
+        c->slab_left -= need;
+        return p;
+    }
+    if (cudaMalloc(&p, need) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
@@ -350,18 +373,6 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
                                              "below dx / 1.5");
     }
     const size_t cells = (size_t)nx * ny * nz, nodes = (size_t)nx * ny * (nz + 1);
-    std::vector<int> cell_ng(cells, 0), cell_g(cells * kMaxG, 0);
-    for (int g = 0; g < grains->n; ++g)
-        for (int dk = -1; dk <= 1; ++dk)
-            for (int dj = -1; dj <= 1; ++dj)
-                for (int di = -1; di <= 1; ++di) {
-                    const int i = (gcell[3 * g] + di + nx) % nx, j = (gcell[3 * g + 1] + dj + ny) % ny,
-                              k = gcell[3 * g + 2] + dk;
-                    const size_t ci = ((size_t)k * ny + j) * nx + i;
-                    if (cell_ng[ci] >= kMaxG) return fail(nullptr, PIC_EINVAL, "grains: more than 8 per MD cell");
-                    cell_g[ci * kMaxG + cell_ng[ci]++] = g;
-                }
-
     pic_ctx* c = new (std::nothrow) pic_ctx();
     if (!c) return fail(nullptr, PIC_ENOMEM, "host allocation");
     c->nx = nx; c->ny = ny; c->nz = nz; c->dx = mesh->dx;
@@ -404,6 +415,13 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
 
     const bool mixed = c->prec == PIC_MIXED;
     const size_t psz = mixed ? sizeof(float4) : sizeof(double4);
+    // slabs: a few per run of a small one (about 128 bytes per node and 4 psz per
+    // particle are held), 64 MB at most, so that what a slab leaves unused stays
+    // small beside the run's memory
+    {
+        const size_t held = 128 * nodes + 2 * psz * (size_t)(c->cap[0] + c->cap[1]), mb2 = (size_t)2 << 20;
+        c->slab_bytes = (std::min(held / 2, (size_t)64 << 20) + mb2 - 1) / mb2 * mb2;
+    }
     bool ok = true;
     for (int sp = 0; sp < 2; ++sp) {
         c->pos[sp] = dev_alloc(c, psz * c->cap[sp]);
@@ -535,6 +553,22 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         return fail(nullptr, PIC_ECUDA, "push window size");
     }
 
+    // ---- the MD cells' grain lists, built on the device from the grains' cells
+    gcell.resize(3 * (size_t)ng1, 0);
+    {
+        cudaError_t e = cudaMemcpyAsync(c->gcell, gcell.data(), sizeof(int) * gcell.size(), cudaMemcpyHostToDevice,
+                                        c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+        if (e == cudaSuccess) e = launch_cell_lists(c, c->d_err);
+        int over = 0;
+        if (c->ng > kMaxG && e == cudaSuccess) {   // (fewer grains cannot overfill a cell)
+            e = cudaMemcpyAsync(&over, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        }
+        if (e != cudaSuccess) { destroy(c); return cuda_fail(nullptr, e, "grain cells"); }
+        if (over) { destroy(c); return fail(nullptr, PIC_EINVAL, "grains: more than 8 per MD cell"); }
+    }
+
     // ---- upload inputs
     // The caller's particle arrays are converted into the run's records on the
     // device (k_stage_particles, which also checks them).  Where the device reads
@@ -552,12 +586,11 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         const bool direct = pma && ats && !(run->flags & PIC_F_STAGE_COPY);
         const int64_t nmax = std::max(run->n[0], run->n[1]);
         const int64_t chunk = direct ? nmax : std::min<int64_t>(nmax, (int64_t)1 << 24);
-        unsigned int* flags = nullptr;   // [bad, largest id]
+        unsigned int* flags = (unsigned int*)c->d_cnt;   // [bad, largest id], until the counters are cleared below
         double* sx = nullptr;
         double* sv = nullptr;
         uint32_t* sid = nullptr;
-        cudaError_t e = cudaMalloc(&flags, 2 * sizeof(unsigned int));
-        if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned int), c->stream);
+        cudaError_t e = cudaMemsetAsync(flags, 0, 2 * sizeof(unsigned int), c->stream);
         if (e == cudaSuccess && !direct) e = cudaMalloc(&sx, 3 * sizeof(double) * (size_t)chunk);
         if (e == cudaSuccess && !direct) e = cudaMalloc(&sv, 3 * sizeof(double) * (size_t)chunk);
         if (e == cudaSuccess && !direct) e = cudaMalloc(&sid, sizeof(uint32_t) * (size_t)chunk);
@@ -585,7 +618,6 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         unsigned int hf[2] = {0, 0};
         if (e == cudaSuccess) e = cudaMemcpyAsync(hf, flags, sizeof hf, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        cudaFree(flags);
         cudaFree(sx);
         cudaFree(sv);
         cudaFree(sid);
@@ -607,7 +639,6 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         grad[g] = grains->radius_host[g];
         gr2[g] = (float)((grad[g] / mesh->dx) * (grad[g] / mesh->dx));
     }
-    gcell.resize(3 * ng1, 0);
     cudaError_t e = cudaSuccess;
     auto up = [&](void* d, const void* h, size_t b) {
         if (e == cudaSuccess && b) e = cudaMemcpy(d, h, b, cudaMemcpyHostToDevice);
@@ -618,11 +649,8 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     up(c->xs32, xs32.data(), sizeof(float) * xs32.size());
     up(c->gpos, gpos.data(), sizeof(double) * gpos.size());
     up(c->grad, grad.data(), sizeof(double) * grad.size());
-    up(c->gcell, gcell.data(), sizeof(int) * gcell.size());
     up(c->goff32, goff.data(), sizeof(float) * goff.size());
     up(c->gr2_32, gr2.data(), sizeof(float) * gr2.size());
-    up(c->cell_ng, cell_ng.data(), sizeof(int) * cells);
-    up(c->cell_g, cell_g.data(), sizeof(int) * cells * kMaxG);
     if (e == cudaSuccess) e = cudaMemset(c->d_cnt, 0, PIC_C_N * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_step, 0, sizeof(uint32_t));

@@ -730,30 +730,46 @@ __global__ void k_grains(Geo g, int ng, double qw, const unsigned long long* gab
     }
 }
 
-// E of the current phi on the 4x4x4 nodes of grain gi's region (unit-charge table)
-__global__ void k_grain_table(int nx, int ny, int nz, double dx, const double* phi, const int* gcell, int gi,
-                              double* tab)
+// The grains of each MD cell (the 3 x 3 x 3 cells around a grain's own, periodic in x
+// and y), in grain order.  A thread per grain and cell claims the cell's next entry;
+// the first to come leaves its grain's complement, by which the second kernel knows
+// the one thread that sorts the cell's at most 8 entries.  On the host the tables of
+// 64 x 64 x 128 cells took 0.4 ms to fill and 0.2 ms to copy.
+__device__ __forceinline__ size_t list_cell(int nx, int ny, const int* gcell, int g, int o)
 {
-    const int t = threadIdx.x;
-    if (t >= 64) return;
-    const int li = t % 4, lj = (t / 4) % 4, lk = t / 16;
-    const int i = ((gcell[3 * gi] - 1 + li) % nx + nx) % nx;
-    const int j = ((gcell[3 * gi + 1] - 1 + lj) % ny + ny) % ny;
-    const int k = gcell[3 * gi + 2] - 1 + lk;
-    const size_t P = (size_t)nx * ny;
-    const size_t n = (size_t)k * P + (size_t)j * nx + i;
-    const double h2 = 2.0 * dx;
-    const size_t row = (size_t)k * P + (size_t)j * nx;
-    double* o = tab + ((size_t)gi * 64 + t) * 3;
-    o[0] = (phi[row + (i + nx - 1) % nx] - phi[row + (i + 1) % nx]) / h2;
-    o[1] = (phi[(size_t)k * P + (size_t)((j + ny - 1) % ny) * nx + i] -
-            phi[(size_t)k * P + (size_t)((j + 1) % ny) * nx + i]) / h2;
-    if (k == 0)
-        o[2] = ((3.0 * phi[n] - 4.0 * phi[n + P]) + phi[n + 2 * P]) / h2;
-    else if (k == nz)
-        o[2] = ((4.0 * phi[n - P] - 3.0 * phi[n]) - phi[n - 2 * P]) / h2;
-    else
-        o[2] = (phi[n - P] - phi[n + P]) / h2;
+    const int i = (gcell[3 * g] + o % 3 - 1 + nx) % nx, j = (gcell[3 * g + 1] + (o / 3) % 3 - 1 + ny) % ny;
+    return ((size_t)(gcell[3 * g + 2] + o / 9 - 1) * ny + j) * nx + i;
+}
+
+__global__ void k_cell_claim(int ng, int nx, int ny, const int* gcell, int* cell_ng, int* cell_g, int* over)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 27LL * ng) return;
+    const int g = (int)(t / 27);
+    const size_t c = list_cell(nx, ny, gcell, g, (int)(t % 27));
+    const int at = atomicAdd(cell_ng + c, 1);
+    if (at < kMaxG) cell_g[c * kMaxG + at] = at == 0 ? ~g : g;
+    else *over = 1;
+}
+
+__global__ void k_cell_order(int ng, int nx, int ny, const int* gcell, const int* cell_ng, int* cell_g)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= 27LL * ng) return;
+    const int g = (int)(t / 27);
+    const size_t c = list_cell(nx, ny, gcell, g, (int)(t % 27));
+    int* l = cell_g + c * kMaxG;
+    if (l[0] != ~g) return;
+    const int n = min(cell_ng[c], kMaxG);
+    int v[kMaxG];
+    v[0] = g;
+    for (int a = 1; a < n; ++a) {
+        const int x = l[a];
+        int b = a;
+        for (; b > 0 && v[b - 1] > x; --b) v[b] = v[b - 1];
+        v[b] = x;
+    }
+    for (int a = 0; a < n; ++a) l[a] = v[a];
 }
 
 // The unit-charge tables by superposition: the mesh is periodic in x and y,
@@ -763,8 +779,8 @@ __global__ void k_grain_table(int nx, int ny, int nz, double dx, const double* p
 // x, y and z around the node.  A grain's unit charge is its CIC deposit on the 8
 // corners of its cell (the weights of k_grains, summing to 2^42), so its
 // potential near the grain is the weighted sum of the 8 corners' moved blocks,
-// and k_grain_table_sup takes its table from that sum with the differences of
-// k_grain_table.
+// and k_grain_table_sup takes its table from that sum with central
+// differences (one-sided second-order ones on the electrodes).
 constexpr int kGreenR = 3, kGreenW = 2 * kGreenR + 1;
 constexpr int kGreenThreads = 512;
 
@@ -1199,11 +1215,16 @@ void launch_grains(pic_ctx* c)
     c->launches += 1;
 }
 
-void launch_grain_table(pic_ctx* c, int gi)
+cudaError_t launch_cell_lists(pic_ctx* c, int* over)
 {
-    k_grain_table<<<1, 64, 0, c->stream>>>(c->nx, c->ny, c->nz, c->dx, c->phi, c->gcell, gi, c->gtab);
-    c->launches += 1;
+    cudaError_t e = cudaMemsetAsync(c->cell_ng, 0, sizeof(int) * c->cells, c->stream);
+    if (e != cudaSuccess || c->ng == 0) return e;
+    const unsigned grid = (unsigned)((27 * (int64_t)c->ng + 127) / 128);
+    k_cell_claim<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g, over);
+    k_cell_order<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g);
+    return cudaGetLastError();
 }
+
 void launch_green_blocks(pic_ctx* c, const int* planes, int n, double* blk)
 {
     if (n == 0) return;

@@ -300,6 +300,8 @@ struct pic_ctx {
     pic_status pending = PIC_OK;
     std::string err;
     std::vector<void*> allocs;
+    char* slab = nullptr;                    // the rest of the newest slab (dev_alloc)
+    size_t slab_left = 0, slab_bytes = 0;
 };
 
 namespace pic {
@@ -312,7 +314,6 @@ void launch_children64(pic_ctx* c);
 void launch_deposit64(pic_ctx* c);
 void launch_moments64(pic_ctx* c);
 void launch_grains(pic_ctx* c);                  // Q from counts, grain CIC into rq
-void launch_grain_table(pic_ctx* c, int g);      // E of phi on grain g's 4x4x4 region nodes
 // the initial plasma of species sp drawn from the seed (ids id0 ..), either layout
 void launch_init_plasma(pic_ctx* c, int sp, int64_t n, uint32_t id0, double t_ev);
 void launch_green_blocks(pic_ctx* c, const int* planes, int n, double* blk);   // phi near a unit charge on (0, 0, planes[q])
@@ -332,6 +333,7 @@ void launch_moments32(pic_ctx* c);
 void launch_moments_phi(pic_ctx* c);
 
 // sort.cu
+cudaError_t launch_cell_lists(pic_ctx* c, int* over);  // cell_ng, cell_g; *over set where a cell has more than 8
 void sort_particles(pic_ctx* c, int sp);
 bool sort_swaps(const pic_ctx* c, int sp);            // whether a sort leaves the species in its other buffers
 void count_live(pic_ctx* c);                         // live records of both species into d_live
