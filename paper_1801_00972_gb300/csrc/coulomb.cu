@@ -10,14 +10,24 @@
 //   k_coul_scatter slot indices grouped by cell, with the pairing key
 //                  (Philox word of (id, step, purpose 6), then id) and the cell
 //   k_coul_rank    one thread per grouped particle: its rank among its cell's
-//                  keys puts the group in key order
+//                  keys puts the group's velocity records in key order (into the
+//                  sort's other buffers, which are free between sorts)
 //   k_coul_like    one thread per like pair (the triplet of an odd group on
 //                  one thread, in order): e-e and Ar+-Ar+ collisions
 //   k_coul_unlike  one thread per particle of the smaller group of a cell: its
-//                  e-Ar+ collisions in the order of the larger group
+//                  e-Ar+ collisions in the order of the larger group; each
+//                  particle's last collision puts its record back in its slot
 // (both stage their work items per warp in shared memory, so that warps run full)
 // Every particle meets its partners in the same order as in a cell-by-cell
 // loop, so the results are those of that loop.
+//
+// The pass is bound by single-record accesses and by the instructions of a
+// collision (two Philox blocks, a logarithm, the rotation).  In key order a pair's
+// records lie side by side, so a record is read out of its slot and put back in it
+// once per step, not once per collision: on 64 x 64 x 256 cells with 5e6 particles
+// of each species k_coul_like 263 -> 181 and k_coul_unlike 260 -> 241 us, k_coul_rank
+// 76 -> 95 us for the reads.  (Records written in the scatter already cost it 45 us
+// more per species; four passes' loads in flight together changed neither kernel.)
 //
 // Pairing: like particles (0,1), (2,3), ...; an odd count's first three form
 // the triplet (0,1), (1,2), (2,0) at half the time step.  Unlike: every
@@ -181,6 +191,76 @@ __device__ void coul_pair64(double* va, double* vb, double fa, double fb, double
 // The same steps with reciprocals and reciprocal square roots in place of the
 // divisions and square roots (a few ulp; the pass is compared with the oracle
 // statistically, not bit for bit).
+
+// The two accepted trials of a collision's stream, the first for the deflection
+// and the second for the azimuth: trials are pairs of words, two per Philox block,
+// taken with 0 < s < 1 (at most 128 for each).  The first four are judged without
+// a branch: a loop per trial runs as often as the slowest of a warp's 32 lanes
+// needs, about four times, with the draw's bookkeeping each time.  One collision in
+// thirty goes on to further blocks.
+struct Trials {
+    uint2 w0, w1;        // the words of the first and of the second accepted trial
+    bool has0, has1;
+    static __device__ __forceinline__ float side(uint32_t w) { return 2.f * u01f(w) - 1.f; }
+    // a^2 + b^2, its roundings written out: one product unrounded for the deflection,
+    // whose logarithm takes it, both rounded for the azimuth, which takes a^2 - b^2 too
+    static __device__ __forceinline__ float radius2_fused(float a, float b) { return __fmaf_rn(a, a, __fmul_rn(b, b)); }
+    static __device__ __forceinline__ float radius2(float a, float b)
+    {
+        return __fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b));
+    }
+    static __device__ __forceinline__ bool first(uint32_t x, uint32_t y)
+    {
+        const float s = radius2_fused(side(x), side(y));
+        return s < 1.f && s > 0.f;
+    }
+    static __device__ __forceinline__ bool second(uint32_t x, uint32_t y)
+    {
+        const float s = radius2(side(x), side(y));
+        return s < 1.f && s > 0.f;
+    }
+    __device__ __forceinline__ Trials(uint32_t id, uint32_t step, uint32_t purpose, uint2 key)
+    {
+        uint4 ctr = make_uint4(id, step, purpose, 0u);
+        const uint4 p = philox4x32_10(ctr, key);
+        ctr.w = 1u;
+        const uint4 q = philox4x32_10(ctr, key);
+        const bool i0 = first(p.x, p.y), i1 = first(p.z, p.w), i2 = first(q.x, q.y), i3 = first(q.z, q.w);
+        has0 = i0 || i1 || i2 || i3;
+        // the second: trial 1 after 0, trial 2 after one of 0, 1, trial 3 after one of 0, 1, 2
+        const bool j1 = i0 && second(p.z, p.w), j2 = (i0 || i1) && second(q.x, q.y);
+        has1 = j1 || j2 || ((i0 || i1 || i2) && second(q.z, q.w));
+        w0 = make_uint2(i0 ? p.x : i1 ? p.z : i2 ? q.x : q.z, i0 ? p.y : i1 ? p.w : i2 ? q.y : q.w);
+        w1 = make_uint2(j1 ? p.z : j2 ? q.x : q.z, j1 ? p.w : j2 ? q.y : q.w);
+        if (!has1) {
+            int stage = has0 ? 1 : 0, t = i0 ? 3 : i1 ? 2 : i2 ? 1 : i3 ? 0 : 4;
+            while (stage < 2) {
+                ctr.w += 1u;
+                const uint4 r = philox4x32_10(ctr, key);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (stage == 2) break;
+                    const uint2 w = h == 0 ? make_uint2(r.x, r.y) : make_uint2(r.z, r.w);
+                    const bool ok = stage == 0 ? first(w.x, w.y) : second(w.x, w.y);
+                    if (ok && stage == 0) {
+                        w0 = w;
+                        has0 = true;
+                    }
+                    if (ok && stage == 1) {
+                        w1 = w;
+                        has1 = true;
+                    }
+                    t += 1;
+                    if (ok || t == 128) {
+                        stage += 1;
+                        t = 0;
+                    }
+                }
+            }
+        }
+    }
+};
+
 __device__ void coul_pair32(float* va, float* vb, float fa, float fb, float cfac, float n, float dtf, uint32_t id,
                             uint32_t step, uint32_t purpose, uint2 pkey)
 {
@@ -190,34 +270,17 @@ __device__ void coul_pair32(float* va, float* vb, float fa, float fb, float cfac
     const float ru = rsqrtf(u2);
     const float um = u2 * ru;
     const float sig2 = ((cfac * n) * dtf) * (ru * ru * ru);
-    PairStream r(id, step, purpose, pkey);
-    float g = 0.f;
-    for (int t = 0; t < 128; ++t) {
-        const uint2 w = r.next();
-        const float a = 2.f * u01f(w.x) - 1.f;
-        const float b = 2.f * u01f(w.y) - 1.f;
-        const float s = a * a + b * b;
-        if (s < 1.f && s > 0.f) {
-            g = a * sqrtf(__fdividef(-2.f * logf(s), s));
-            break;
-        }
-    }
+    const Trials r(id, step, purpose, pkey);
+    const float a0 = Trials::side(r.w0.x), s0 = Trials::radius2_fused(a0, Trials::side(r.w0.y));
+    const float g = r.has0 ? a0 * sqrtf(__fdividef(-2.f * logf(s0), s0)) : 0.f;
     const float d = sqrtf(sig2) * g;
     const float rden = __fdividef(1.f, 1.f + d * d);
     const float sn = 2.f * d * rden, omc = 2.f * d * d * rden;
-    float a = 0.f, b = 0.f, s2 = 0.f;
-    int t;
-    for (t = 0; t < 128; ++t) {
-        const uint2 w = r.next();
-        a = 2.f * u01f(w.x) - 1.f;
-        b = 2.f * u01f(w.y) - 1.f;
-        s2 = a * a + b * b;
-        if (s2 < 1.f && s2 > 0.f) break;
-    }
     float cp = 1.f, sp = 0.f;
-    if (t < 128) {
-        const float rs = __fdividef(1.f, s2);
-        cp = (a * a - b * b) * rs;
+    if (r.has1) {
+        const float a = Trials::side(r.w1.x), b = Trials::side(r.w1.y);
+        const float rs = __fdividef(1.f, Trials::radius2(a, b));
+        cp = __fsub_rn(__fmul_rn(a, a), __fmul_rn(b, b)) * rs;
         sp = 2.f * a * b * rs;
     }
     const float up2 = u[0] * u[0] + u[1] * u[1];
@@ -241,7 +304,9 @@ __device__ void coul_pair32(float* va, float* vb, float fa, float fb, float cfac
 }
 
 struct CoulArgs {
-    void* vel[2];
+    void* vel[2];                 // the run's records
+    void* rec[2];                 // the same in key order, cell by cell
+    const unsigned int* slot[2];  // where each of those belongs
     double w, vol, dt;            // weight, cell volume, step
     double cf[3];                 // e-e, i-i, e-i: q^4 lnL / (8 pi eps0^2 mu^2) (SI); mixed: times dt / (dx/dt)^3
     double fac[2][2];             // mu / m_a of a pair of species (a, b), mu = m_a m_b / (m_a + m_b)
@@ -274,37 +339,26 @@ __device__ __forceinline__ X pick(const X (&v)[3], int k)
     return k == 0 ? v[0] : k == 1 ? v[1] : v[2];
 }
 
-// one collision of slot qa (species sa, the pair's first particle) with slot qb
-// (species sb); kind 0 e-e, 1 i-i, 2 e-i.  Whole records are read and written
-// back; their fourth word (the id) passes through.
-__device__ __forceinline__ void collide(const CoulArgs& a, int sa, unsigned int qa, int sb, unsigned int qb,
-                                        int kind, double dens, bool half, uint32_t step, uint32_t purpose, double*)
+// one collision of record A (species sa, the pair's first particle) with B (species
+// sb); kind 0 e-e, 1 i-i, 2 e-i.  The records' fourth word (the id) stays.
+__device__ __forceinline__ void collide(const CoulArgs& a, int sa, double4& A, int sb, double4& B, int kind,
+                                        double dens, bool half, uint32_t step, uint32_t purpose)
 {
-    double4* pa = reinterpret_cast<double4*>(sa == 0 ? a.vel[0] : a.vel[1]) + qa;
-    double4* pb = reinterpret_cast<double4*>(sb == 0 ? a.vel[0] : a.vel[1]) + qb;
-    double4 A = *pa, B = *pb;
     double va[3] = {A.x, A.y, A.z}, vb[3] = {B.x, B.y, B.z};
     const double dt = half ? 0.5 * a.dt : a.dt;
     coul_pair64(va, vb, pick(a.fac, sa, sb), pick(a.fac, sb, sa), pick(a.cf, kind), dens, dt, coul_id(A), step,
                 purpose, a.pkey);
     A.x = va[0]; A.y = va[1]; A.z = va[2];
     B.x = vb[0]; B.y = vb[1]; B.z = vb[2];
-    *pa = A;
-    *pb = B;
 }
-__device__ __forceinline__ void collide(const CoulArgs& a, int sa, unsigned int qa, int sb, unsigned int qb,
-                                        int kind, float dens, bool half, uint32_t step, uint32_t purpose, float*)
+__device__ __forceinline__ void collide(const CoulArgs& a, int sa, float4& A, int sb, float4& B, int kind,
+                                        float dens, bool half, uint32_t step, uint32_t purpose)
 {
-    float4* pa = reinterpret_cast<float4*>(sa == 0 ? a.vel[0] : a.vel[1]) + qa;
-    float4* pb = reinterpret_cast<float4*>(sb == 0 ? a.vel[0] : a.vel[1]) + qb;
-    float4 A = *pa, B = *pb;
     float va[3] = {A.x, A.y, A.z}, vb[3] = {B.x, B.y, B.z};
     coul_pair32(va, vb, pick(a.fac32, sa, sb), pick(a.fac32, sb, sa), pick(a.cf32, kind), dens, half ? 0.5f : 1.f,
                 coul_id(A), step, purpose, a.pkey);
     A.x = va[0]; A.y = va[1]; A.z = va[2];
     B.x = vb[0]; B.y = vb[1]; B.z = vb[2];
-    *pa = A;
-    *pb = B;
 }
 
 struct CoulGroups {
@@ -328,11 +382,14 @@ __device__ __forceinline__ void group_of(const CoulGroups& g, int sp, unsigned i
     b1 = e[c];
 }
 
-// rank of each grouped particle's key among its cell's keys -> key order
+// rank of each grouped particle's key among its cell's keys -> records and slots
+// in key order
+template <typename T4>
 __global__ void __launch_bounds__(256) k_coul_rank(const CoulGroups g, const unsigned long long* key_e,
                                                    const unsigned long long* key_i, const unsigned int* idx_e,
-                                                   const unsigned int* idx_i, unsigned int* ord_e,
-                                                   unsigned int* ord_i)
+                                                   const unsigned int* idx_i, const T4* __restrict__ vel_e,
+                                                   const T4* __restrict__ vel_i, unsigned int* ord_e,
+                                                   unsigned int* ord_i, T4* __restrict__ out_e, T4* __restrict__ out_i)
 {
     unsigned int n0, n1;
     group_totals(g, n0, n1);
@@ -342,12 +399,15 @@ __global__ void __launch_bounds__(256) k_coul_rank(const CoulGroups g, const uns
         const int sp = t < n0 ? 0 : 1;
         const unsigned int d = (unsigned int)(sp == 0 ? t : t - n0);
         const unsigned long long* key = sp == 0 ? key_e : key_i;
+        const unsigned int slot = (sp == 0 ? idx_e : idx_i)[d];
+        const T4 v = (sp == 0 ? vel_e : vel_i)[slot];
         unsigned int b0, b1;
         group_of(g, sp, (sp == 0 ? g.cell[0] : g.cell[1])[d], b0, b1);
         const unsigned long long k = key[d];
         unsigned int r = 0;
         for (unsigned int j = b0; j < b1; ++j) r += key[j] < k;     // keys are unique (they end with the id)
-        (sp == 0 ? ord_e : ord_i)[b0 + r] = (sp == 0 ? idx_e : idx_i)[d];
+        (sp == 0 ? ord_e : ord_i)[b0 + r] = slot;
+        (sp == 0 ? out_e : out_i)[b0 + r] = v;
     }
 }
 
@@ -409,12 +469,10 @@ struct WarpQueue {
 
 // like pairs: in a group of n in key order, (0,1), (2,3), ... for even n; for
 // odd n the triplet (0,1), (1,2), (2,0) at half the step, then (3,4), (5,6), ...
-// An item is (group start, position of its first particle, n, species | stage
-// << 1): stage 0 a pair, 1..3 the triplet's collisions in order.
-template <typename T>
-__global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_like(const CoulArgs a, const CoulGroups g,
-                                                                  const unsigned int* ord_e,
-                                                                  const unsigned int* ord_i)
+// An item is (its first particle, 0, n, species | stage << 1): stage 0 a pair, 1..3
+// the triplet's collisions in order.
+template <typename T, typename T4>
+__global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_like(const CoulArgs a, const CoulGroups g)
 {
     __shared__ uint4 store[kWarps][64];
     const uint32_t step = *a.step - 1u;
@@ -425,11 +483,14 @@ __global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_like(const CoulArgs
     auto one = [&](uint4& it) -> bool {
         const int sp = (int)(it.w & 1u);
         const unsigned int stage = it.w >> 1;
-        const unsigned int* L = (sp == 0 ? ord_e : ord_i) + it.x;
-        const unsigned int ib = stage == 0u ? it.y + 1u : stage == 3u ? 0u : stage;
-        const unsigned int ia = stage == 0u ? it.y : stage - 1u;
-        collide(a, sp, L[ia], sp, L[ib], sp, density(a, it.z, (T*)nullptr), stage != 0u, step,
-                sp == 0 ? kPurCoulEE : kPurCoulII, (T*)nullptr);
+        T4* r = reinterpret_cast<T4*>(sp == 0 ? a.rec[0] : a.rec[1]) + it.x;
+        T4* pa = r + (stage == 0u ? 0u : stage - 1u);
+        T4* pb = r + (stage == 0u ? 1u : stage == 3u ? 0u : stage);
+        T4 A = *pa, B = *pb;
+        collide(a, sp, A, sp, B, sp, density(a, it.z, (T*)nullptr), stage != 0u, step,
+                sp == 0 ? kPurCoulEE : kPurCoulII);
+        *pa = A;
+        *pb = B;
         it.w += 2u;
         return stage == 1u || stage == 2u;
     };
@@ -447,7 +508,7 @@ __global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_like(const CoulArgs
             if (n >= 2) {
                 const bool trip = n % 2 == 1 && r == 0;
                 has = trip || (n % 2 == 1 ? (r >= 3 && (r & 1) == 1) : (r & 1) == 0);
-                v = make_uint4(b0, r, n, (unsigned int)sp | (trip ? 2u : 0u));
+                v = make_uint4(d, 0u, n, (unsigned int)sp | (trip ? 2u : 0u));
             }
         }
         q.push(has, v);
@@ -458,12 +519,11 @@ __global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_like(const CoulArgs
 
 // e-Ar+: every particle of the larger group A (electrons on a tie) meets
 // B[k mod |B|] at the density of B; the item of B's position b takes
-// k = b, b + |B|, ... in that order.  An item is (the ord index of A[k], B's
-// slot, |B| | A's species << 31, collisions left).
-template <typename T>
-__global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_unlike(const CoulArgs a, const CoulGroups g,
-                                                                    const unsigned int* ord_e,
-                                                                    const unsigned int* ord_i)
+// k = b, b + |B|, ... in that order.  An item is (A[k], its B, |B| | A's species
+// << 31, collisions left).  Each particle goes back to its slot with its last
+// collision, or at once where its cell has none of the other species.
+template <typename T, typename T4>
+__global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_unlike(const CoulArgs a, const CoulGroups g)
 {
     __shared__ uint4 store[kWarps][64];
     const uint32_t step = *a.step - 1u;
@@ -472,13 +532,19 @@ __global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_unlike(const CoulAr
     const unsigned long long total = (unsigned long long)n0 + n1;
     WarpQueue q{store[threadIdx.x >> 5], 0u};
     auto one = [&](uint4& it) -> bool {
-        const int big = (int)(it.z >> 31);
+        const bool ions = (it.z >> 31) != 0u;   // whether A is the ions
         const unsigned int nb = it.z & 0x7fffffffu;
-        const unsigned int qa = (big == 0 ? ord_e : ord_i)[it.x];
-        collide(a, big, qa, 1 - big, it.y, 2, density(a, nb, (T*)nullptr), false, step, kPurCoulEI, (T*)nullptr);
+        T4* pb = reinterpret_cast<T4*>(ions ? a.rec[0] : a.rec[1]) + it.y;
+        T4 A = reinterpret_cast<const T4*>(ions ? a.rec[1] : a.rec[0])[it.x], B = *pb;
+        const unsigned int to = (ions ? a.slot[1] : a.slot[0])[it.x];
+        const bool more = it.w > 1u;
+        if (!more) pb = reinterpret_cast<T4*>(ions ? a.vel[0] : a.vel[1]) + (ions ? a.slot[0] : a.slot[1])[it.y];
+        collide(a, ions ? 1 : 0, A, ions ? 0 : 1, B, 2, density(a, nb, (T*)nullptr), false, step, kPurCoulEI);
+        reinterpret_cast<T4*>(ions ? a.vel[1] : a.vel[0])[to] = A;
+        *pb = B;
         it.x += nb;
         it.w -= 1u;
-        return it.w != 0u;
+        return more;
     };
     PIC_COUL_WARP_LOOP(total)
     {
@@ -498,9 +564,10 @@ __global__ void __launch_bounds__(256, PIC_COUL_MINB) k_coul_unlike(const CoulAr
             if (has) {
                 const unsigned int na = big == 0 ? ne : ni, nb = big == 0 ? ni : ne;
                 const unsigned int b = d - (sp == 0 ? e0 : i0);
-                const unsigned int qb = (sp == 0 ? ord_e : ord_i)[d];
-                v = make_uint4((big == 0 ? e0 : i0) + b, qb, nb | ((unsigned int)big << 31),
-                               (na - b + nb - 1u) / nb);
+                v = make_uint4((big == 0 ? e0 : i0) + b, d, nb | ((unsigned int)big << 31), (na - b + nb - 1u) / nb);
+            } else if (ne == 0 || ni == 0) {
+                reinterpret_cast<T4*>(sp == 0 ? a.vel[0] : a.vel[1])[(sp == 0 ? a.slot[0] : a.slot[1])[d]] =
+                    reinterpret_cast<const T4*>(sp == 0 ? a.rec[0] : a.rec[1])[d];
             }
         }
         q.push(has, v);
@@ -541,7 +608,10 @@ void PIC_COUL_LAUNCH(pic_ctx* c)
                                                          sp, c->cs_end[sp], c->cs_idx[sp], c->cs_key[sp],
                                                          c->cs_cell[sp], c->nx, c->ny, c->d_step, c->key);
         c->launches += 2;
+        // (the sort's other buffers are free between sorts)
         a.vel[sp] = c->vel[sp];
+        a.rec[sp] = c->pos_alt[sp];
+        a.slot[sp] = c->cs_ord[sp];
     }
     a.w = c->W;
     a.vol = c->dx * c->dx * c->dx;
@@ -574,10 +644,11 @@ void PIC_COUL_LAUNCH(pic_ctx* c)
     // the collision kernels: one resident wave, so that each warp's queue runs
     // many full rounds before its last, partial ones
     const int gridc = std::min(grid, 152 * PIC_COUL_MINB);
-    k_coul_rank<<<grid, 256, 0, c->stream>>>(g, c->cs_key[0], c->cs_key[1], c->cs_idx[0], c->cs_idx[1],
-                                             c->cs_ord[0], c->cs_ord[1]);
-    k_coul_like<CT><<<gridc, 256, 0, c->stream>>>(a, g, c->cs_ord[0], c->cs_ord[1]);
-    k_coul_unlike<CT><<<gridc, 256, 0, c->stream>>>(a, g, c->cs_ord[0], c->cs_ord[1]);
+    k_coul_rank<CT4><<<grid, 256, 0, c->stream>>>(g, c->cs_key[0], c->cs_key[1], c->cs_idx[0], c->cs_idx[1],
+                                                  (const CT4*)c->vel[0], (const CT4*)c->vel[1], c->cs_ord[0],
+                                                  c->cs_ord[1], (CT4*)c->pos_alt[0], (CT4*)c->pos_alt[1]);
+    k_coul_like<CT, CT4><<<gridc, 256, 0, c->stream>>>(a, g);
+    k_coul_unlike<CT, CT4><<<gridc, 256, 0, c->stream>>>(a, g);
     c->launches += 3;
 }
 
