@@ -93,9 +93,8 @@ pic_status cuda_fail(pic_ctx* c, cudaError_t e, const char* what)
     return fail(c, PIC_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-// zero every moment window (rf average, phase bins, fine grid) on `st`
-// (synchronous memsets when st is null)
-cudaError_t clear_moments(pic_ctx* c, cudaStream_t st)
+// zero every moment window (rf average, phase bins, fine grid) on the run's stream
+cudaError_t clear_moments(pic_ctx* c)
 {
     const size_t nb = (size_t)c->nph;
     const size_t sz[10] = {sizeof(double) * 4 * c->nodes * nb, sizeof(double) * 4 * c->nodes * nb,
@@ -107,7 +106,7 @@ cudaError_t clear_moments(pic_ctx* c, cudaStream_t st)
                    c->mom32[0], c->mom32[1]};
     cudaError_t e = cudaSuccess;
     for (int q = 0; q < 10 && e == cudaSuccess; ++q)
-        if (p[q]) e = st ? cudaMemsetAsync(p[q], 0, sz[q], st) : cudaMemset(p[q], 0, sz[q]);
+        if (p[q]) e = cudaMemsetAsync(p[q], 0, sz[q], c->stream);
     return e;
 }
 
@@ -248,6 +247,7 @@ void drop_events(pic_ctx* c);
 void destroy(pic_ctx* c)
 {
     if (!c) return;
+    cudaStreamSynchronize(c->stream);
     drop_events(c);
     for (cudaGraphExec_t g : {c->g_pre, c->g_push[0], c->g_push[1], c->g_solve, c->g_post[0][0], c->g_post[0][1],
                               c->g_post[1][0], c->g_post[1][1], c->g_mom[0], c->g_mom[1]})
@@ -281,7 +281,6 @@ const char* pic_last_error(const pic_ctx* ctx) { return ctx ? ctx->err.c_str() :
 
 void pic_destroy(pic_ctx* ctx)
 {
-    if (ctx) cudaStreamSynchronize(ctx->stream);
     destroy(ctx);
 }
 
@@ -553,6 +552,16 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         return fail(nullptr, PIC_ECUDA, "push window size");
     }
 
+    // The clears and copies up to here went to the legacy default stream, whose
+    // copies to the device may return before they are done and which a
+    // non-blocking stream does not wait for.  From here on everything goes to the
+    // run's own stream; the host arrays live until it is synchronised (by the last
+    // check below, or by destroy).
+    {
+        const cudaError_t e = cudaStreamSynchronize(nullptr);
+        if (e != cudaSuccess) { destroy(c); return cuda_fail(nullptr, e, "setup"); }
+    }
+
     // ---- the MD cells' grain lists, built on the device from the grains' cells
     gcell.resize(3 * (size_t)ng1, 0);
     {
@@ -641,7 +650,10 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     }
     cudaError_t e = cudaSuccess;
     auto up = [&](void* d, const void* h, size_t b) {
-        if (e == cudaSuccess && b) e = cudaMemcpy(d, h, b, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && b) e = cudaMemcpyAsync(d, h, b, cudaMemcpyHostToDevice, c->stream);
+    };
+    auto clear = [&](void* d, size_t b) {
+        if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, b, c->stream);
     };
     up(c->d_nslot, nslot, sizeof nslot);
     up(c->d_next_id, &next_id, sizeof next_id);
@@ -651,29 +663,28 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     up(c->grad, grad.data(), sizeof(double) * grad.size());
     up(c->goff32, goff.data(), sizeof(float) * goff.size());
     up(c->gr2_32, gr2.data(), sizeof(float) * gr2.size());
-    if (e == cudaSuccess) e = cudaMemset(c->d_cnt, 0, PIC_C_N * sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(c->d_step, 0, sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(c->d_iters, 0, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemset(c->d_res, 0, sizeof(double));
-    if (e == cudaSuccess) e = cudaMemset(c->d_solve_flag, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(c->d_iter_total, 0, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(c->d_vb_last, 0, sizeof(double));
+    clear(c->d_cnt, PIC_C_N * sizeof(unsigned long long));
+    clear(c->d_err, sizeof(int));
+    clear(c->d_step, sizeof(uint32_t));
+    clear(c->d_iters, sizeof(unsigned int));
+    clear(c->d_res, sizeof(double));
+    clear(c->d_solve_flag, sizeof(int));
+    clear(c->d_iter_total, sizeof(unsigned long long));
+    clear(c->d_vb_last, sizeof(double));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->aux2, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMemset(c->d_nch, 0, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(c->gabs, 0, sizeof(unsigned long long) * 2 * ng1);
-    if (e == cudaSuccess) e = cudaMemset(c->gq, 0, sizeof(double) * ng1);
-    if (e == cudaSuccess) e = cudaMemset(c->gq32, 0, sizeof(float) * ng1);
-    if (e == cudaSuccess) e = cudaMemset(c->phi, 0, sizeof(double) * nodes);
+    clear(c->d_nch, sizeof(unsigned long long));
+    clear(c->gabs, sizeof(unsigned long long) * 2 * ng1);
+    clear(c->gq, sizeof(double) * ng1);
+    clear(c->gq32, sizeof(float) * ng1);
+    clear(c->phi, sizeof(double) * nodes);
     if (e == cudaSuccess && (c->flags & PIC_F_MOMENTS)) {
-        e = cudaMemset(c->d_bin, 0, sizeof(int));
-        if (e == cudaSuccess) e = clear_moments(c, nullptr);
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        clear(c->d_bin, sizeof(int));
+        if (e == cudaSuccess) e = clear_moments(c);
     }
     if (e == cudaSuccess && t_ev) {
         // electrons take ids 0 .. n_e - 1, ions n_e .. n_e + n_i - 1
@@ -689,6 +700,7 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     // and y, so a unit charge on node (i, j, k) gives the same potential moved by
     // (i, j)); each grain's table is then the sum of its 8 corners' moved
     // potentials with its CIC weights (launch_grain_tables_sup)
+    std::vector<float> tab32;
     {
         std::vector<int> plane((size_t)nz + 1, -1), planes;
         for (int g = 0; g < c->ng; ++g)
@@ -708,7 +720,8 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
             eg = cudaMalloc(&blk, sizeof(double) * 343 * planes.size());
             if (eg == cudaSuccess) eg = cudaMalloc(&dplane, sizeof(int) * plane.size());
             if (eg == cudaSuccess)
-                eg = cudaMemcpy(dplane, plane.data(), sizeof(int) * plane.size(), cudaMemcpyHostToDevice);
+                eg = cudaMemcpyAsync(dplane, plane.data(), sizeof(int) * plane.size(), cudaMemcpyHostToDevice,
+                                     c->stream);
             if (eg == cudaSuccess) {
                 launch_green_blocks(c, dplane + nz + 1, np, blk);
                 launch_grain_tables_sup(c, blk, dplane);
@@ -722,10 +735,10 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         std::vector<double> tab(kTab * (size_t)ng1);
         e = cudaMemcpyAsync(tab.data(), c->gtab, sizeof(double) * tab.size(), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        std::vector<float> tab32(tab.size());
+        tab32.resize(tab.size());
         for (size_t i = 0; i < tab.size(); ++i) tab32[i] = (float)tab[i];
-        if (e == cudaSuccess) e = cudaMemcpy(c->gtab32, tab32.data(), sizeof(float) * tab32.size(),
-                                             cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(c->gtab32, tab32.data(), sizeof(float) * tab32.size(),
+                                                  cudaMemcpyHostToDevice, c->stream);
         if (e != cudaSuccess) { destroy(c); return cuda_fail(nullptr, e, "grain tables"); }
     }
 
@@ -1592,7 +1605,7 @@ pic_status pic_moments(pic_ctx* c, int32_t what, double* out, size_t len, int32_
     k = moments_window(c, what, 0, c->nph, c->msteps, out);
     if (k != PIC_OK) return k;
     if (reset) {
-        const cudaError_t e = clear_moments(c, c->stream);
+        const cudaError_t e = clear_moments(c);
         if (e != cudaSuccess) return cuda_fail(c, e, "moments reset");
         c->msteps = 0;
     }
