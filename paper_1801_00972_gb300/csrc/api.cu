@@ -372,6 +372,20 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
                                              "below dx / 1.5");
     }
     const size_t cells = (size_t)nx * ny * nz, nodes = (size_t)nx * ny * (nz + 1);
+    if (grains->n > kMaxG) {
+        // the cells of every grain's MD region, sorted: a cell of more than kMaxG
+        // regions comes again kMaxG places further on
+        std::vector<size_t> md;
+        md.reserve(27 * (size_t)grains->n);
+        for (int g = 0; g < grains->n; ++g)
+            for (int q = 0; q < 27; ++q) {
+                const int i = (gcell[3 * g] + q % 3 - 1 + nx) % nx, j = (gcell[3 * g + 1] + q / 3 % 3 - 1 + ny) % ny;
+                md.push_back(((size_t)(gcell[3 * g + 2] + q / 9 - 1) * ny + j) * nx + i);
+            }
+        std::sort(md.begin(), md.end());
+        for (size_t q = 0; q + kMaxG < md.size(); ++q)
+            if (md[q] == md[q + kMaxG]) return fail(nullptr, PIC_EINVAL, "grains: more than 8 per MD cell");
+    }
     pic_ctx* c = new (std::nothrow) pic_ctx();
     if (!c) return fail(nullptr, PIC_ENOMEM, "host allocation");
     c->nx = nx; c->ny = ny; c->nz = nz; c->dx = mesh->dx;
@@ -567,15 +581,8 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     {
         cudaError_t e = cudaMemcpyAsync(c->gcell, gcell.data(), sizeof(int) * gcell.size(), cudaMemcpyHostToDevice,
                                         c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
-        if (e == cudaSuccess) e = launch_cell_lists(c, c->d_err);
-        int over = 0;
-        if (c->ng > kMaxG && e == cudaSuccess) {   // (fewer grains cannot overfill a cell)
-            e = cudaMemcpyAsync(&over, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        }
+        if (e == cudaSuccess) e = launch_cell_lists(c);
         if (e != cudaSuccess) { destroy(c); return cuda_fail(nullptr, e, "grain cells"); }
-        if (over) { destroy(c); return fail(nullptr, PIC_EINVAL, "grains: more than 8 per MD cell"); }
     }
 
     // ---- upload inputs

@@ -731,17 +731,18 @@ __global__ void k_grains(Geo g, int ng, double qw, const unsigned long long* gab
 }
 
 // The grains of each MD cell (the 3 x 3 x 3 cells around a grain's own, periodic in x
-// and y), in grain order.  A thread per grain and cell claims the cell's next entry;
-// the first to come leaves its grain's complement, by which the second kernel knows
-// the one thread that sorts the cell's at most 8 entries.  On the host the tables of
-// 64 x 64 x 128 cells took 0.4 ms to fill and 0.2 ms to copy.
+// and y), in grain order; at most kMaxG, as the caller has checked.  A thread per
+// grain and cell claims the cell's next entry; the first to come leaves its grain's
+// complement, by which the second kernel knows the one thread that sorts the cell's
+// entries.  On the host the tables of 64 x 64 x 128 cells took 0.4 ms to fill and
+// 0.2 ms to copy.
 __device__ __forceinline__ size_t list_cell(int nx, int ny, const int* gcell, int g, int o)
 {
     const int i = (gcell[3 * g] + o % 3 - 1 + nx) % nx, j = (gcell[3 * g + 1] + (o / 3) % 3 - 1 + ny) % ny;
     return ((size_t)(gcell[3 * g + 2] + o / 9 - 1) * ny + j) * nx + i;
 }
 
-__global__ void k_cell_claim(int ng, int nx, int ny, const int* gcell, int* cell_ng, int* cell_g, int* over)
+__global__ void k_cell_claim(int ng, int nx, int ny, const int* gcell, int* cell_ng, int* cell_g)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 27LL * ng) return;
@@ -749,7 +750,6 @@ __global__ void k_cell_claim(int ng, int nx, int ny, const int* gcell, int* cell
     const size_t c = list_cell(nx, ny, gcell, g, (int)(t % 27));
     const int at = atomicAdd(cell_ng + c, 1);
     if (at < kMaxG) cell_g[c * kMaxG + at] = at == 0 ? ~g : g;
-    else *over = 1;
 }
 
 __global__ void k_cell_order(int ng, int nx, int ny, const int* gcell, const int* cell_ng, int* cell_g)
@@ -1215,12 +1215,12 @@ void launch_grains(pic_ctx* c)
     c->launches += 1;
 }
 
-cudaError_t launch_cell_lists(pic_ctx* c, int* over)
+cudaError_t launch_cell_lists(pic_ctx* c)
 {
     cudaError_t e = cudaMemsetAsync(c->cell_ng, 0, sizeof(int) * c->cells, c->stream);
     if (e != cudaSuccess || c->ng == 0) return e;
     const unsigned grid = (unsigned)((27 * (int64_t)c->ng + 127) / 128);
-    k_cell_claim<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g, over);
+    k_cell_claim<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g);
     k_cell_order<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g);
     return cudaGetLastError();
 }

@@ -333,7 +333,7 @@ void launch_moments32(pic_ctx* c);
 void launch_moments_phi(pic_ctx* c);
 
 // sort.cu
-cudaError_t launch_cell_lists(pic_ctx* c, int* over);  // cell_ng, cell_g; *over set where a cell has more than 8
+cudaError_t launch_cell_lists(pic_ctx* c);             // cell_ng, cell_g
 void sort_particles(pic_ctx* c, int sp);
 bool sort_swaps(const pic_ctx* c, int sp);            // whether a sort leaves the species in its other buffers
 void count_live(pic_ctx* c);                         // live records of both species into d_live
