@@ -205,7 +205,7 @@ pic_status check(pic_ctx* c)
     e = cudaMemcpy(&sf, c->d_solve_flag, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(c, e, "solve flag");
     if (sf != 0) {
-        cudaMemset(c->d_solve_flag, 0, sizeof(int));
+        cudaMemsetAsync(c->d_solve_flag, 0, sizeof(int), c->stream);
         if (sf == PIC_ENONFINITE) return fail(c, PIC_ENONFINITE, "Poisson solve: non-finite residual");
         return fail(c, PIC_ENOTCONV, "Poisson solve did not reach the tolerance within max_cycles");
     }
@@ -1521,8 +1521,10 @@ pic_status pic_set_grain_table(pic_ctx* c, const double* tab, size_t len)
     if (k != PIC_OK || !len) return k;
     std::vector<float> t32(len);
     for (size_t i = 0; i < len; ++i) t32[i] = (float)tab[i];
-    cudaError_t e = cudaMemcpy(c->gtab, tab, sizeof(double) * len, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(c->gtab32, t32.data(), sizeof(float) * len, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpyAsync(c->gtab, tab, sizeof(double) * len, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->gtab32, t32.data(), sizeof(float) * len, cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     return e == cudaSuccess ? PIC_OK : cuda_fail(c, e, "table copy");
 }
 
@@ -1534,7 +1536,8 @@ pic_status pic_set_grain_counts(pic_ctx* c, const int64_t* n_abs, size_t len)
     if (len) {
         for (size_t i = 0; i < len; ++i)
             if (n_abs[i] < 0) return fail(c, PIC_EINVAL, "negative count");
-        const cudaError_t e = cudaMemcpy(c->gabs, n_abs, sizeof(int64_t) * len, cudaMemcpyHostToDevice);
+        cudaError_t e = cudaMemcpyAsync(c->gabs, n_abs, sizeof(int64_t) * len, cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "count copy");
     }
     cudaMemsetAsync(c->rq, 0, sizeof(unsigned long long) * c->nodes, c->stream);

@@ -27,3 +27,20 @@ def test_start_of_a_run_is_ordered(recorder, prec, kw, drawn):  # noqa: F811
         run.close()
     assert sum(c[0] == "launch" and c[1] == str(STREAM) for c in calls) > 10
     assert not unordered(calls)
+
+
+@pytest.mark.parametrize("prec", [P.PIC_MIXED, P.PIC_FP64])
+def test_calls_on_a_run_are_ordered(recorder, prec):  # noqa: F811
+    wl = I.small(nx=16, ny=16, nz=32, grains=3)
+    with recorder.in_place():
+        run = P.Run(wl, None, prec=prec, stream=STREAM, flags=P.PIC_F_MOMENTS | P.PIC_F_NO_GRAPH)
+        calls = {"phi": lambda: run.set_phi(run.phi()), "tables": lambda: run.set_gtab(run.gtab()),
+                 "counts": lambda: run.set_grain_counts([[1, 2], [3, 4], [5, 6]]), "step": lambda: run.step(2),
+                 "moments": lambda: run.moments(1, reset=True), "counters": run.counts,
+                 "tuning": lambda: run.set_tuning(dict(sort_every=3, tile=[4, 4, 4], halo=1, order=0))}
+        for name, call in calls.items():
+            recorder.lib.rec_clear()
+            call()
+            run.advance()   # the run's next kernels
+            assert not unordered(recorder.calls()), name
+        run.close()
