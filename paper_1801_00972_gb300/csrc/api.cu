@@ -457,12 +457,9 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
             ok = ok && c->md_res[sp];
             c->md_list[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * c->cap[sp]);
             c->md_next[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * c->cap[sp]);
-            ok = ok && c->md_list[sp] && c->md_next[sp];
+            c->mcc_list[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * c->cap[sp]);
+            ok = ok && c->md_list[sp] && c->md_next[sp] && c->mcc_list[sp];
         }
-    }
-    for (int sp = 0; sp < 2; ++sp) {
-        c->mcc_list[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * c->cap[sp]);
-        ok = ok && c->mcc_list[sp];
     }
     c->d_lists = (unsigned int*)dev_alloc(c, 6 * sizeof(unsigned int));
     ok = ok && c->d_lists && cudaMemset(c->d_lists, 0, 6 * sizeof(unsigned int)) == cudaSuccess;

@@ -1132,7 +1132,7 @@ void launch_push64(pic_ctx* c)
         p.hm = c->hm[sp];
         const double below = std::ceil(c->pnull[sp] * 0x1p32 - 0.5);   // u + 1/2 < pnull 2^32
         p.null_below = below > 0.0 ? (unsigned long long)below : 0ull;
-        p.mcc_list = c->mcc_list[sp];
+        p.mcc_list = (unsigned int*)c->pos_alt[sp];   // (the sort's other buffers are free between sorts)
         p.mcc_n = c->d_lists + 2 * sp + 1;
         p.nu_max = c->nu_max[sp];
         p.de = c->de[sp];

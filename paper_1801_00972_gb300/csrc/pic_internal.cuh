@@ -177,7 +177,7 @@ struct pic_ctx {
     unsigned int* md_next[2] = {nullptr, nullptr};   // mixed: the same list being built for the next step
     float4* md_res[2] = {nullptr, nullptr};           // mixed: MD results (pos, vel pairs) until the join
     int64_t md_rescap = 0;
-    unsigned int* mcc_list[2] = {nullptr, nullptr};  // slots of collision candidates this step
+    unsigned int* mcc_list[2] = {nullptr, nullptr};  // mixed: slots of collision candidates this step
     unsigned int* d_lists = nullptr;                  // [md_n e, mcc_n e, md_n i, mcc_n i, next_n e, next_n i] (FP64: mcc_n)
 
     // mesh arrays
