@@ -1222,6 +1222,7 @@ cudaError_t launch_cell_lists(pic_ctx* c)
     const unsigned grid = (unsigned)((27 * (int64_t)c->ng + 127) / 128);
     k_cell_claim<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g);
     k_cell_order<<<grid, 128, 0, c->stream>>>(c->ng, c->nx, c->ny, c->gcell, c->cell_ng, c->cell_g);
+    c->launches += 2;
     return cudaGetLastError();
 }
 
