@@ -60,6 +60,10 @@ namespace cg = cooperative_groups;
 
 constexpr int kPre = PIC_MG_PRE;         // pre-smoothing sweeps of a V-cycle
 constexpr int kPost = PIC_MG_POST;       // post-smoothing sweeps
+// the restriction reads red residuals only, the black ones being zero after a
+// sweep, and the prolongation onto a split level leaves the red nodes to the red
+// half-sweep that starts the post-smoothing
+static_assert(kPre >= 1 && kPost >= 1, "a V-cycle needs a sweep before and a sweep after the coarse correction");
 
 struct Dims {
     int nx, ny, nz;
