@@ -554,7 +554,7 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
          c->phi_alt && c->f64 && (c->e32 || c->e64) && c->d_norm && c->xs64 && c->xs32 && c->gpos && c->grad &&
          c->gcell && c->gq && c->gabs && c->gtab && c->gtab32 && c->gq32 && c->goff32 && c->gr2_32 && c->cell_ng &&
          c->cell_g && c->cursor;
-    if (!ok || !sort_scratch_setup(c) || mg_setup(c) != PIC_OK) {
+    if (!ok || !sort_scratch_setup(c, c->nkeys) || mg_setup(c) != PIC_OK) {
         destroy(c);
         return fail(nullptr, PIC_ENOMEM, "device allocation failed");
     }
@@ -1194,24 +1194,21 @@ pic_status pic_set_tuning(pic_ctx* c, const pic_tuning* t)
     for (int a = 0; a < 3; ++a) ntile[a] = (n[a] + t->tile[a] - 1) / t->tile[a];
     const int64_t ntiles = (int64_t)ntile[0] * ntile[1] * ntile[2];
     const size_t nkeys = (size_t)ntiles * (size_t)(t->tile[0] * t->tile[1] * t->tile[2]);
-    if (nkeys > c->nkeys_cap || ntiles > c->ntiles_cap) {
-        unsigned int* cur = nkeys > c->nkeys_cap ? (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (nkeys + 1))
-                                                 : c->cursor;
-        unsigned int* ts0 = ntiles > c->ntiles_cap ? (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (ntiles + 1))
-                                                   : c->tstart[0];
-        unsigned int* ts1 = ntiles > c->ntiles_cap ? (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (ntiles + 1))
-                                                   : c->tstart[1];
-        unsigned char* md = ntiles > c->ntiles_cap ? (unsigned char*)dev_alloc(c, (size_t)ntiles) : c->tile_md;
-        if (!cur || !ts0 || !ts1 || !md) return fail(c, PIC_ENOMEM, "tuning: key buffers");
+    if (nkeys > c->nkeys_cap) {
+        unsigned int* cur = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (nkeys + 1));
+        if (!cur || !sort_scratch_setup(c, nkeys)) return fail(c, PIC_ENOMEM, "tuning: key buffers");
         c->cursor = cur;
-        c->tile_md = md;
+        c->nkeys_cap = nkeys;
+    }
+    if (ntiles > c->ntiles_cap) {
+        unsigned int* ts0 = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (ntiles + 1));
+        unsigned int* ts1 = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (ntiles + 1));
+        unsigned char* md = (unsigned char*)dev_alloc(c, (size_t)ntiles);
+        if (!ts0 || !ts1 || !md) return fail(c, PIC_ENOMEM, "tuning: tile buffers");
         c->tstart[0] = ts0;
         c->tstart[1] = ts1;
-        c->nkeys_cap = std::max(c->nkeys_cap, nkeys);
-        c->ntiles_cap = std::max(c->ntiles_cap, ntiles);
-        const size_t old_keys = c->nkeys;
-        c->nkeys = nkeys;
-        if (nkeys > old_keys && !sort_scratch_setup(c)) return fail(c, PIC_ENOMEM, "tuning: scan scratch");
+        c->tile_md = md;
+        c->ntiles_cap = ntiles;
     }
     for (int a = 0; a < 3; ++a) { c->tile[a] = t->tile[a]; c->ntile[a] = ntile[a]; }
     c->ntiles = ntiles;

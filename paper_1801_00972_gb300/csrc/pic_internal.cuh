@@ -237,7 +237,6 @@ struct pic_ctx {
                                                     // (ntiles + 1 entries; the last = particles sorted)
     unsigned char* tile_md = nullptr;               // mixed: 1 where a tile's deposit window holds an MD cell
     std::vector<unsigned int*> scan_tmp;
-    std::vector<size_t> scan_len;
 
     // multigrid
     std::vector<pic::MGLevel> mg;
@@ -349,7 +348,7 @@ void launch_oml(pic_ctx* c, int with_cx, double* out);   // 6 values per grain f
 void launch_coulomb(pic_ctx* c);                    // binary Coulomb collisions of the step's particles
 void launch_coulomb_fp64(pic_ctx* c);               // (its FP64 unit, built without fused multiply-add)
 void launch_coulomb_mixed(pic_ctx* c);              // (its float unit)
-size_t sort_scratch_setup(pic_ctx* c);
+bool sort_scratch_setup(pic_ctx* c, size_t nkeys);   // scan scratch for up to nkeys sort keys
 
 // poisson.cu
 pic_status mg_setup(pic_ctx* c);

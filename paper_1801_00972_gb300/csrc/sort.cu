@@ -302,25 +302,22 @@ unsigned int* scan(pic_ctx* c, unsigned int* data, size_t n, int level)
 
 void scan_cells(pic_ctx* c, unsigned int* data) { scan(c, data, c->cells, 0); }
 
-// scratch: one block-sum buffer per scan level, plus a final total slot
-// (sized for the sort keys, which are at least as many as the cells)
-size_t sort_scratch_setup(pic_ctx* c)
+// scratch: one block-sum buffer per scan level, for a key range of nkeys and for the
+// cells (of the Coulomb pass).  Shorter ranges use the same buffers, so a caller
+// asks anew only for a range longer than all before it; the old ones stay where the
+// new cannot be had.
+bool sort_scratch_setup(pic_ctx* c, size_t nkeys)
 {
-    size_t n = std::max(c->nkeys, c->cells);
-    size_t bytes = 0;
-    c->scan_tmp.clear();
-    c->scan_len.clear();
-    while (true) {
-        const size_t nb = (n + kScanBlock - 1) / kScanBlock;
-        unsigned int* p = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (nb + 1));
-        if (!p) return 0;
-        c->scan_tmp.push_back(p);
-        c->scan_len.push_back(nb);
-        bytes += sizeof(unsigned int) * (nb + 1);
-        if (nb <= 1) break;
-        n = nb;
+    std::vector<unsigned int*> tmp;
+    for (size_t n = std::max(nkeys, c->cells);;) {
+        n = (n + kScanBlock - 1) / kScanBlock;
+        unsigned int* p = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * n);
+        if (!p) return false;
+        tmp.push_back(p);
+        if (n <= 1) break;
     }
-    return bytes + 1;
+    c->scan_tmp = tmp;
+    return true;
 }
 
 void count_live(pic_ctx* c)
