@@ -151,7 +151,9 @@ typedef struct {
  * host's page tables (a coherent CPU-GPU link), else copied in chunks of 2^24
  * particles; a particle outside the box or non-finite gives PIC_EINVAL after
  * the device has checked it (the other arguments are checked first, on the
- * host). */
+ * host).  A run with grains on a mesh whose coarsest solver level converges too
+ * slowly (narrow meshes whose long axis does not halve, e.g. 8 x 8 x 301)
+ * gives PIC_ENOTCONV. */
 pic_status pic_init(const pic_mesh* mesh, const pic_electrodes* el, const pic_gas* gas,
                     const pic_grains* grains, const pic_run* run, void* cuda_stream,
                     pic_ctx** out);

@@ -563,6 +563,15 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
         return fail(nullptr, PIC_ECUDA, "push window size");
     }
 
+    // A few meshes, narrow ones whose long axis does not halve, leave a coarsest level
+    // on which the cycles barely converge.  A run with grains is refused there: where
+    // 200 cycles from a unit charge (whose share of the slowest mode is
+    // sqrt(2 / (nx ny nz)) at most) leave more than 1e-12 of it.
+    if (c->ng > 0 && std::sqrt(2.0 / (double)cells) * std::pow(mg_slowest(c), 200.0) > 1e-12) {
+        destroy(c);
+        return fail(nullptr, PIC_ENOTCONV, "grain fields: the field solve converges too slowly on this mesh");
+    }
+
     // The clears and copies up to here went to the legacy default stream, whose
     // copies to the device may return before they are done and which a
     // non-blocking stream does not wait for.  From here on everything goes to the

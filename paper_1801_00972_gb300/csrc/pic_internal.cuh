@@ -352,6 +352,7 @@ bool sort_scratch_setup(pic_ctx* c, size_t nkeys);   // scan scratch for up to n
 
 // poisson.cu
 pic_status mg_setup(pic_ctx* c);
+double mg_slowest(const pic_ctx* c);   // factor of the slowest error per cycle (0: solved exactly)
 void launch_rhs(pic_ctx* c, double scale, double v_bot, double v_top, bool warm_shift);
 void phi_sync_f64(pic_ctx* c);       // mixed: write the FP64 copy of the potential
 void phi_from_f64(pic_ctx* c);       // mixed: potential from the FP64 copy

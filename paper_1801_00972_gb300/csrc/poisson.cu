@@ -1173,6 +1173,13 @@ __global__ void __launch_bounds__(kClThreads) k_vcycle_cluster(const ClusterLeve
 
 constexpr size_t kClSmemMax = 220 * 1024;
 
+// red-black sweeps of a coarsest level that has no exact solve
+int coarse_sweeps(const MGLevel& L)
+{
+    const int m = std::max(std::max(L.nx, L.ny), L.nz);
+    return std::min(4 * m * m + 16, 2000);
+}
+
 // layout of the levels l0.. for a cluster of C CTAs; false if it does not fit
 template <typename T>
 bool cluster_levels(const pic_ctx* c, int l0, int C, ClusterLevels<T>* out, size_t* smem)
@@ -1211,9 +1218,7 @@ bool cluster_levels(const pic_ctx* c, int l0, int C, ClusterLevels<T>* out, size
     L.gu = (T*)c->mg[l0].u;
     L.gf = (const T*)c->mg[l0].f;
     L.ainv = (const T*)c->coarse_inv;
-    const MGLevel& Cl = c->mg.back();
-    const int m = std::max(std::max(Cl.nx, Cl.ny), Cl.nz);
-    L.sweeps = std::min(4 * m * m + 16, 2000);
+    L.sweeps = coarse_sweeps(c->mg.back());
     if (off > kClSmemMax) return false;
     if (out) *out = L;
     if (smem) *smem = off;
@@ -2553,6 +2558,16 @@ pic_status mg_setup(pic_ctx* c)
             return PIC_ECUDA;
     }
     return PIC_OK;
+}
+
+// What one cycle leaves of the slowest error, the half sine in z that is constant in
+// x and y: the smoothers above hardly touch it, and where the coarsest level is
+// swept, each sweep multiplies it by ((4 + 2 cos(pi / nz)) / 6)^2.  0: solved exactly.
+double mg_slowest(const pic_ctx* c)
+{
+    const MGLevel& L = c->mg.back();
+    if (c->ex_level >= 0 || c->coarse_inv || L.nz < 2) return 0.0;
+    return std::pow((4.0 + 2.0 * std::cos(kPI / L.nz)) / 6.0, 2.0 * coarse_sweeps(L));
 }
 
 void launch_rhs(pic_ctx* c, double scale, double v_bot, double v_top, bool warm_shift)

@@ -43,3 +43,21 @@ def test_clusters_are_refused_by_their_fullest_cell(recorder, shape, most):  # n
         seen.add(full)
         assert _status(recorder, pos, shape) == (P.PIC_EINVAL if full > 8 else P.PIC_ENOMEM), (n, full)
     assert {8, 9} <= seen   # both sides of the limit came up
+
+
+@pytest.mark.parametrize("shape,refused", [((8, 8, 301), True), ((8, 8, 401), True), ((10, 6, 331), True), ((8, 8, 221), False),
+                                           ((8, 8, 151), False), ((8, 8, 450), False), ((16, 16, 49), False),
+                                           ((16, 16, 32), False), ((80, 48, 100), False), ((4, 4, 63), False)])
+def test_meshes_whose_solve_barely_converges_take_no_grains(recorder, shape, refused):  # noqa: F811
+    # 8 x 8 x 301: a unit charge's solve on the device stood above 1e-12 after 200 cycles; 8 x 8 x 221
+    # reached it, 8 x 8 x 450 halves to a level that is solved exactly
+    wl = I.small(nx=shape[0], ny=shape[1], nz=shape[2], grains=1)
+    bare = dataclasses.replace(wl, grain_pos=np.zeros((0, 3)), grain_r=np.zeros(0))
+    with recorder.in_place():
+        P.Run(bare, None, stream=STREAM).close()
+        if refused:
+            with pytest.raises(P.PicError) as e:
+                P.Run(wl, None, stream=STREAM)
+            assert e.value.status == P.PIC_ENOTCONV
+        else:
+            P.Run(wl, None, stream=STREAM).close()
