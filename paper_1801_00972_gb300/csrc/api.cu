@@ -1582,7 +1582,7 @@ pic_status pic_profile_read(pic_ctx* c, double* push_ms, int64_t* push_launches,
     const cudaError_t e = cudaMemcpy(&tot, c->d_iter_total, sizeof tot, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(c, e, "iteration counter");
     if (push_ms) *push_ms = t[0];
-    if (push_launches) *push_launches = (int64_t)c->ev_push.size() * 2;   // one launch per species
+    if (push_launches) *push_launches = (int64_t)c->ev_push.size() * 2;   // one per species and step
     if (solve_ms) *solve_ms = t[1];
     if (solves) *solves = (int64_t)c->ev_solve.size();
     if (solve_iterations) *solve_iterations = (int64_t)(tot - c->prof_iter0);

@@ -167,11 +167,6 @@ __device__ __forceinline__ double exact_double(unsigned long long n)
     const int e = 63 - __clzll((long long)n);
     return n ? __longlong_as_double((long long)(((unsigned long long)(1022 + e) << 52) + (n << (52 - e)))) : 0.0;
 }
-__device__ __forceinline__ double exact_double32(unsigned int n)   // n < 2^20: the high word alone
-{
-    const int e = 31 - __clz((int)n);
-    return n ? __hiloint2double((int)(((unsigned int)(1022 + e) << 20) + (n << (20 - e))), 0) : 0.0;
-}
 // a whole number 0 <= v < 2^32
 __device__ __forceinline__ unsigned int exact_uint(double v)
 {

@@ -319,6 +319,7 @@ void launch_green_blocks(pic_ctx* c, const int* planes, int n, double* blk);   /
 void launch_grain_tables_sup(pic_ctx* c, const double* blk, const int* plane);   // every grain's table from them
 void launch_stage_particles(pic_ctx* c, int sp, const double* x, const double* v, const uint32_t* id, int64_t n,
                             int64_t q0, unsigned int* bad, unsigned int* max_id);   // caller particles into records
+cudaError_t launch_cell_lists(pic_ctx* c);       // cell_ng, cell_g
 
 // particles_mixed.cu
 void launch_efield32(pic_ctx* c);
@@ -332,7 +333,6 @@ void launch_moments32(pic_ctx* c);
 void launch_moments_phi(pic_ctx* c);
 
 // sort.cu
-cudaError_t launch_cell_lists(pic_ctx* c);             // cell_ng, cell_g
 void sort_particles(pic_ctx* c, int sp);
 bool sort_swaps(const pic_ctx* c, int sp);            // whether a sort leaves the species in its other buffers
 void count_live(pic_ctx* c);                         // live records of both species into d_live
