@@ -503,6 +503,8 @@ pic_status init_run(const pic_mesh* mesh, const pic_electrodes* el, const pic_ga
     c->cursor = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (c->nkeys + 1));
     c->nkeys_cap = c->nkeys;
     c->ntiles_cap = c->ntiles;
+    for (int sp = 0; sp < 2; ++sp) c->n_first[sp] = run->n[sp];
+    c->two_pass = two_passes_pay(c);
     if (mixed)
         for (int sp = 0; sp < 2; ++sp) {
             c->tstart[sp] = (unsigned int*)dev_alloc(c, sizeof(unsigned int) * (size_t)(c->ntiles + 1));
@@ -1083,6 +1085,18 @@ void drop_graphs(pic_ctx* c)
         }
 }
 
+// a new sort interval; the step graphs go where the electrons' sort takes another
+// route with it (returns whether)
+bool set_sort_every(pic_ctx* c, int32_t s)
+{
+    c->sort_every = s;
+    const bool two = two_passes_pay(c);
+    if (two == c->two_pass) return false;
+    cudaStreamSynchronize(c->stream);
+    drop_graphs(c);
+    c->two_pass = two;
+    return true;
+}
 
 size_t tuning_window_bytes(const int32_t tile[3], int32_t halo)
 {
@@ -1137,11 +1151,12 @@ pic_status pic_tune_sort(pic_ctx* c, int32_t steps_per_candidate, int32_t* chose
     float best_ms = 0.f;
     pic_status st = PIC_OK;
     for (int32_t s : cand) {
-        c->sort_every = s;
+        const bool rebuild = set_sort_every(c, s);
         const int32_t whole = std::max(steps_per_candidate, 2 * s);
         const int32_t n = (whole + s - 1) / s * s;
-        // start on a sort boundary so that every candidate covers whole periods
-        const int32_t lead = (int32_t)((s - c->step % s) % s);
+        // start on a sort boundary so that every candidate covers whole periods (two
+        // periods ahead where the step graphs, of both parities, have to be built)
+        const int32_t lead = (int32_t)((s - c->step % s) % s) + (rebuild ? 2 * s : 0);
         if (lead > 0 && (st = step_enqueue(c, lead)) != PIC_OK) break;
         cudaEventRecord(e0, c->stream);
         if ((st = step_enqueue(c, n)) != PIC_OK) break;
@@ -1157,7 +1172,7 @@ pic_status pic_tune_sort(pic_ctx* c, int32_t steps_per_candidate, int32_t* chose
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    c->sort_every = best;
+    set_sort_every(c, best);
     if (chosen) *chosen = best;
     return st;
 }
@@ -1190,10 +1205,13 @@ pic_status pic_set_tuning(pic_ctx* c, const pic_tuning* t)
     if (tuning_window_bytes(t->tile, t->halo) > kMaxWindowBytes)
         return fail(c, PIC_EINVAL, "tuning: the deposit window (tile + 1 + 2 halo nodes per axis, 8 B each) "
                                    "exceeds 96 KB");
-    c->sort_every = t->sort_every;
     const bool same = t->tile[0] == c->tile[0] && t->tile[1] == c->tile[1] && t->tile[2] == c->tile[2] &&
                       t->halo == c->halo && t->order == c->sort_order;
-    if (same) return PIC_OK;
+    if (same) {
+        set_sort_every(c, t->sort_every);
+        return PIC_OK;
+    }
+    c->sort_every = t->sort_every;
     // new sort keys: wait for queued work, size the key buffers, re-sort both
     // species now (the tile ranges must describe the new order), drop the step
     // graphs (grid and window size are baked into them)
@@ -1224,6 +1242,7 @@ pic_status pic_set_tuning(pic_ctx* c, const pic_tuning* t)
     c->nkeys = nkeys;
     c->halo = t->halo;
     c->sort_order = t->order;
+    c->two_pass = two_passes_pay(c);
     e = push32_set_window(c);
     if (e != cudaSuccess) return cuda_fail(c, e, "tuning: push window size");
     drop_graphs(c);
@@ -1255,10 +1274,12 @@ pic_status pic_tune(pic_ctx* c, int32_t steps_per_candidate, const char* cache_p
     // ms per step of one candidate over whole sort periods, after a warm-up period
     pic_status st = PIC_OK;
     auto time_it = [&](const pic_tuning& t, float* ms) -> pic_status {
+        const bool two = c->two_pass;
         pic_status r = pic_set_tuning(c, &t);
         if (r != PIC_OK) return r;
         const int32_t s = t.sort_every;
-        const int32_t lead = (int32_t)((s - c->step % s) % s) + s;
+        // (two periods where a new interval has the step graphs rebuilt, one of each parity)
+        const int32_t lead = (int32_t)((s - c->step % s) % s) + (c->two_pass != two ? 2 * s : s);
         if ((r = step_enqueue(c, lead)) != PIC_OK) return r;
         const int32_t n = (std::max(steps_per_candidate, 2 * s) + s - 1) / s * s;
         cudaEventRecord(e0, c->stream);

@@ -159,6 +159,7 @@ struct pic_ctx {
     cudaStream_t stream;
     int64_t step;
     int64_t cap[2];
+    int64_t n_first[2] = {0, 0};             // particles at the start
     int64_t child_cap;
 
     // particles: fp64 double4 {x,y,z,cell} / {vx,vy,vz,id}; mixed float4 {ox,oy,oz,cell bits} / {v (cells/step), id bits}
@@ -232,6 +233,7 @@ struct pic_ctx {
     int ntile[3] = {1, 1, 1};                // mixed: tiles per axis
     int64_t ntiles = 0;
     int halo = 2;                            // mixed: deposit window margin around a tile, in cells
+    bool two_pass = false;                   // electrons' cell order in two passes (two_passes_pay)
     int sort_order = 0;                      // mixed sort keys: 0 by cell inside the tile, 1 by tile only
     unsigned int* tstart[2] = {nullptr, nullptr};   // mixed: first slot of each tile after the last sort
                                                     // (ntiles + 1 entries; the last = particles sorted)
@@ -334,6 +336,7 @@ void launch_moments_phi(pic_ctx* c);
 
 // sort.cu
 void sort_particles(pic_ctx* c, int sp);
+bool two_passes_pay(const pic_ctx* c);               // whether the tiling, count and interval favour two passes
 bool sort_swaps(const pic_ctx* c, int sp);            // whether a sort leaves the species in its other buffers
 void count_live(pic_ctx* c);                         // live records of both species into d_live
 void scan_cells(pic_ctx* c, unsigned int* data);   // exclusive scan of one value per cell, in place

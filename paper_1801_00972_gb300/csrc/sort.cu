@@ -2,8 +2,8 @@
 // dropping dead slots.  The FP64 path sorts by linear cell index; the mixed
 // path by tile (blocks of tile[0] x tile[1] x tile[2] cells, tile-major, the
 // cells of a tile row-major inside it), so that each tile's particles occupy
-// one contiguous slot range, which the push hands to one thread block; the
-// electrons' order by cell is made in two passes (sort_swaps).  The
+// one contiguous slot range, which the push hands to one thread block; where that
+// pays the electrons' order by cell is made in two passes (two_passes_pay).  The
 // order of particles inside a cell is not fixed (atomic scatter); nothing in a
 // step depends on it: the deposit is an exact integer sum and the random
 // numbers are keyed on particle ids.
@@ -215,7 +215,7 @@ __global__ void k_tile_ranges(const unsigned int* cursor, unsigned int* tstart, 
 // a permutation (reads scattered inside the tile's few ten KB, writes in whole
 // lines), more of them written to their places directly.
 constexpr int kOrderThreads = 256;
-constexpr int kOrderCells = 4096;   // largest tile, in cells
+constexpr int kOrderCells = 1024;   // largest tile, in cells
 constexpr int kPermMax = 8192;
 
 __global__ void __launch_bounds__(kOrderThreads) k_order_cells(const float4* __restrict__ pos, const float4* __restrict__ vel,
@@ -333,7 +333,7 @@ void count_live(pic_ctx* c)
     c->launches += 2;
 }
 
-// Electrons in cell order take two passes: by tile, then by cell inside each
+// Electrons in cell order can take two passes: by tile, then by cell inside each
 // tile.  They cross about a third of a cell per step and axis, so a few steps after
 // a sort a tile's electrons are spread over three times its cells: a scatter
 // straight to cells is 32 separate 16-byte writes per warp and nearly one
@@ -341,17 +341,36 @@ void count_live(pic_ctx* c)
 // though, and inside a tile the rest is local.  2.5e8 electrons on 256 x 256 x
 // 1024 cells, sorted every 5 steps: histogram 1.6 and scatter 14.8 ms in one
 // pass; 1.1, 3.0 and 3.7 ms in two (16 GB each of records read and written:
-// 2.6 ms is the memory's).  Ions hardly move between
-// sorts: their one pass writes whole lines already (3.4 ms).  Tiles of fewer than
-// 64 cells leave a block of the second pass too little to do, larger ones than
-// kOrderCells do not fit its counters; those take the one pass.
-bool sort_swaps(const pic_ctx* c, int sp)
+// 2.6 ms is the memory's).  Ions hardly move between sorts: their one pass writes
+// whole lines already (3.4 ms).
+//
+// The second pass gives a tile to one block, whatever it holds, so it pays only
+// where many tiles hold a fair number of particles each, and where the electrons
+// have moved.  Particle half of a step with 1 to 2.4e8 electrons, sorted every
+// 5 steps (others in brackets), two passes against one:
+//   tiles (8 x 8 x 8)        131072 0.85  65536 0.88-0.98  16384 0.90-0.95  8192 0.95-0.96
+//                            4096 0.96-1.01 [up to 1.07]  2048 0.98-1.24 [1.66]  16 1.18 [1.89]
+//   4096 tiles, per tile     977: 0.98  2441: 0.96-0.99  4882: 1.00-1.01 [1.07]
+//   16384 tiles, per tile    488: 0.95  6104: 0.90  7019: 0.93  9155 (beyond kPermMax in part): 1.03 [1.41]
+//   cells per tile           64: 1.00 at 122 to 305 a tile, 0.89 at 457 to 763  256: 0.85-0.96
+//                            1024: 0.90-0.98  2048: 1.03-1.16 [1.33]  4096: 1.06-1.19 [1.39]
+//   cells crossed per sort   16384 tiles 0.04: 1.13-1.22  0.36: 1.00-1.14  0.54: 0.98-1.01  0.73: 0.95
+//                            1.8: 0.90-0.95  3.6: 0.95-0.97  7.3: 0.98-1.01; 131072 tiles 0.36: 0.96
+//                            8192 tiles 3.6: 0.96-1.00  7.3: 1.00-1.03
+// `cells crossed` takes electrons of 3 eV, the workloads' temperature; the particle
+// count is the run's first.
+bool two_passes_pay(const pic_ctx* c)
 {
-    const bool two = c->prec == PIC_MIXED && sp == 0 && c->sort_order == 0 &&
-                     c->tile[0] * c->tile[1] * c->tile[2] >= kOrderThreads / 4 &&
-                     c->tile[0] * c->tile[1] * c->tile[2] <= kOrderCells;
-    return !two;
+    if (c->prec != PIC_MIXED || c->sort_order != 0) return false;
+    const double cells = (double)c->tile[0] * c->tile[1] * c->tile[2];
+    const double tiles = (double)c->ntiles, each = (double)c->n_first[0] / tiles;
+    const double crossed = c->sort_every * c->dt * 7.3e5 / c->dx;
+    return cells >= 64 && cells <= kOrderCells && each <= kPermMax * 7 / 8 && each + cells >= 500 &&
+           (tiles >= 8192 || (tiles >= 4096 && each <= 2500)) && crossed >= (tiles >= 65536 ? 0.3 : 0.6) &&
+           crossed <= tiles / 2048;
 }
+
+bool sort_swaps(const pic_ctx* c, int sp) { return !(sp == 0 && c->two_pass); }
 
 void sort_particles(pic_ctx* c, int sp)
 {
