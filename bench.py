@@ -38,12 +38,15 @@ TUNE_STEPS = 12      # steps per candidate of the autotuner (tile shape, window 
 TUNE_CACHE = os.path.join(tempfile.gettempdir(), "pic_tune_cache.json")
 
 
-# Poisson: algorithmic bytes per mesh node per refinement iteration: the
-# V(2,2) cycle (4 red-black sweeps x 12 B + residual/restriction 8.5 B +
-# prolongation 8.5 B, x 8/7 for the coarser levels) plus the refinement's
-# residual and update (40 B)
-BYTES_NODE_MIXED = 74 + 40
-BYTES_NODE_FP64 = 148 + 40
+# Poisson: algorithmic bytes per mesh node per refinement iteration.  The V(2,2) cycle
+# on a red-black split level, in float: 7 half-sweeps of 6 B (the other colour's u and
+# this colour's f read, this colour's u written; the first of the 8 is folded into the
+# second, on coarser levels into the restriction), red residuals 8 B, restriction 2.5 B,
+# prolongation onto the black nodes 4.5 B, x 8/7 for the coarser levels: 65 B; the
+# refinement's residual and update 32 B.  FP64: the same in doubles, the finest level's
+# first half-sweep (8 B) not folded: 138 B, and 40 B.
+BYTES_NODE_MIXED = 65 + 32
+BYTES_NODE_FP64 = 138 + 40
 DIAG_PHASES = 16           # rf phase bins of the diagnostics run
 # committed ncu summary of the push kernel on the headline workload (DRAM traffic per launch)
 PUSH_PROFILE = "k_push32_w4_256x256x1024_5e8.md"
@@ -376,9 +379,9 @@ def push_roofline(res, peak, peak_kind, profile_name):
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
             "bytes_per_particle_step": BYTES_MIXED,
             "traffic": traffic_from_profile("particles_mixed.cu", profile_name) if profile_name else None,
-            "timing": "CUDA events around each step's push phase, in which the electron and ion launches "
-                      "overlap on two streams (the MD-region kernel on a third); achieved = both launches' "
-                      "algorithmic bytes / the phase time",
+            "timing": "CUDA events around each step's push phase: one push launch for both species, the "
+                      "MD-region kernel beside it on a second stream, the collision kernels; achieved = the "
+                      "push's algorithmic bytes / the phase time",
             "phase_ms_per_step": pr["push_ms"] / max(res["steps"], 1),
             "launches": pr["push_launches"]}
 

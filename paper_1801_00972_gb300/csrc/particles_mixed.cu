@@ -9,12 +9,12 @@
 // The push works in cell units: v += (q/m) E dt^2/dx, offset += v, with the
 // integer part carried into the cell.  Collisions convert to SI.
 //
-// One step runs three kernels per species:
+// One step runs three kernels for the particles:
 //   k_push32  every particle outside the MD regions: gather, push, electrode
 //             loss, the null-collision test, deposit.  The particles are
-//             sorted by tile (8 x 8 x 8 cells); one thread block takes the slot
-//             range of one tile as it stood at the last sort and sums its
-//             deposits in a shared-memory window over the tile's nodes plus a
+//             sorted by tile (8 x 8 x 8 cells); one thread block takes both
+//             species' slot ranges of one tile as they stood at the last sort
+//             and sums their deposits in a shared-memory window over the tile's nodes plus a
 //             margin of `halo` cells (particles drift between sorts), flushed
 //             with one global atomic per touched node.  Corners outside the
 //             window, and the ionization products appended since the sort
@@ -24,10 +24,9 @@
 //   k_md32    the MD-region particles (listed during the previous step, so it
 //             runs on a second stream alongside k_push32): Dt/40 substeps with
 //             the PPPM correction, grain absorption, MCC, deposit.
-//   k_mcc32   the collision candidates: process selection and kinematics.
-// The ion push and its collisions run on a third stream beside the electron
-// push: the species share only the charge array and the counters, both summed
-// with atomics, so the overlap hides each launch's last partial wave.
+//             Both species in one launch.
+//   k_mcc32   the collision candidates: process selection and kinematics, one
+//             launch per species, the ions' on a third stream.
 #include <algorithm>
 #include <climits>
 
