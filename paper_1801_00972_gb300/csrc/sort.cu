@@ -348,14 +348,14 @@ void count_live(pic_ctx* c)
 // where many tiles hold a fair number of particles each, and where the electrons
 // have moved.  Particle half of a step with 1 to 2.4e8 electrons, sorted every
 // 5 steps (others in brackets), two passes against one:
-//   tiles (8 x 8 x 8)        131072 0.85  65536 0.88-0.98  16384 0.90-0.95  8192 0.95-0.96
-//                            4096 0.96-1.01 [up to 1.07]  2048 0.98-1.24 [1.66]  16 1.18 [1.89]
+//   tiles (8 x 8 x 8)        131072 0.85  65536 0.88-0.98  16384 0.90-0.99  8192 0.95-0.99
+//                            4096 0.96-1.01 [1.23]  2048 0.98-1.24 [1.66]  16 1.18 [1.89]
 //   4096 tiles, per tile     977: 0.98  2441: 0.96-0.99  4882: 1.00-1.01 [1.07]
 //   16384 tiles, per tile    488: 0.95  6104: 0.90  7019: 0.93  9155 (beyond kPermMax in part): 1.03 [1.41]
 //   cells per tile           64: 1.00 at 122 to 305 a tile, 0.89 at 457 to 763  256: 0.85-0.96
-//                            1024: 0.90-0.98  2048: 1.03-1.16 [1.33]  4096: 1.06-1.19 [1.39]
-//   cells crossed per sort   16384 tiles 0.04: 1.13-1.22  0.36: 1.00-1.14  0.54: 0.98-1.01  0.73: 0.95
-//                            1.8: 0.90-0.95  3.6: 0.95-0.97  7.3: 0.98-1.01; 131072 tiles 0.36: 0.96
+//                            1024: 0.90-0.98 (8192 tiles or more)  2048: 1.03-1.16 [1.33]  4096: 1.06-1.19 [1.39]
+//   cells crossed per sort   16384 tiles 0.04: 1.13-1.22  0.36: 1.00-1.14  0.54: 0.98-1.01  0.73: 0.95-1.00
+//                            1.8: 0.90-0.99  3.6: 0.95-1.00  7.3: 0.98-1.01; 131072 tiles 0.36: 0.96
 //                            8192 tiles 3.6: 0.96-1.00  7.3: 1.00-1.03
 // `cells crossed` takes electrons of 3 eV, the workloads' temperature; the particle
 // count is the run's first.

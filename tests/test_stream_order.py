@@ -8,7 +8,7 @@ from paper_1801_00972_gb300 import inputs as I
 from recording import STREAM, recorder, unordered  # noqa: F401
 
 
-def test_the_checker_sees_a_missing_wait():
+def test_a_missing_wait_is_seen():
     copy = ["copy", "0", "1", "1", "2", "8"]
     assert unordered([copy, ["launch", "5", "k", "1"]])
     assert unordered([["memset", "0", "1", "8"], ["memset", "5", "1", "8"]])
