@@ -218,9 +218,10 @@ typedef struct {
 /* Current choices of a run (out: host). */
 pic_status pic_get_tuning(const pic_ctx* ctx, pic_tuning* out);
 
-/* Apply choices (in: host).  A new tile shape or margin synchronises the
- * run's stream, re-sorts both species at once and rebuilds the step graphs
- * at the next step.  PIC_EINVAL for values out of range. */
+/* Apply choices (in: host).  A new tile shape, margin or order synchronises
+ * the run's stream, re-sorts both species at once and rebuilds the step graphs
+ * at the next step; an interval with which the electrons are sorted another
+ * way (in one pass or two) synchronises and rebuilds them too.  PIC_EINVAL for values out of range. */
 pic_status pic_set_tuning(pic_ctx* ctx, const pic_tuning* t);
 
 /* Autotuner: times candidate choices on the run itself with CUDA events and
